@@ -534,8 +534,7 @@ RICH_API rich_status rich_destroy(rich_ctx *ctx) {
         }
         if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
         if (ctx->up_stream) cudaStreamDestroy(ctx->up_stream);
-        if (ctx->graph_exec) cudaGraphExecDestroy(ctx->graph_exec);
-        if (ctx->graph) cudaGraphDestroy(ctx->graph);
+        drop_graph(ctx);
         if (ctx->capture_stream) cudaStreamDestroy(ctx->capture_stream);
         cudaFree(ctx->d_acc);
         cudaFreeHost(ctx->h_acc);

@@ -111,3 +111,30 @@ def test_chunked_run_resumes_exactly():
     ctx2.close()
     assert int(whole.sum()) > 1000
     assert torch.equal(whole, resumed)
+
+
+def test_contexts_with_graphs_come_and_go():
+    """Each context owns its captured graph and destroys it once: contexts
+    that captured, replayed in turn and were closed leave the graphs of the
+    others, and of contexts made later, in order."""
+    wl = W.batched(6, seed=2)
+
+    def captured():
+        ctx = rich.Context(0)
+        ctx.init_geometry(wl.scene)
+        out = rich.TraceOutputs(200_000, wl.scene.pixels_per_event, 3, 6, 0)
+        ctx.graph_capture(rich.DeviceTracks(wl.tracks), out, wl.n_minus_1, seed=wl.seed)
+        return ctx, out
+
+    counts = []
+    held = [captured() for _ in range(3)]
+    for _ in range(3):
+        for ctx, out in held:
+            out.clear()
+            ctx.graph_launch()
+            counts.append(ctx.hits()[0])
+        held.pop(0)[0].close()
+        held.append(captured())
+    for ctx, _ in held:
+        ctx.close()
+    assert counts[0] > 0 and len(set(counts)) == 1
