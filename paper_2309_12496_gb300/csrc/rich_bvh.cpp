@@ -277,11 +277,22 @@ bool build_bvh(const float *vertices, const int32_t *surface, int64_t n_tris, Bv
     std::vector<int> items, weight;
     std::vector<std::pair<int32_t, int>> group_root;   // (surface id, root in all)
     all.reserve(2 * (size_t)n_tris + 2 * groups.size());
+    // the groups are independent: built on a few host threads, joined in order
+    std::vector<std::pair<Builder, int>> built;
+    built.reserve(groups.size());
     for (auto &[sid, tris] : groups) {
-        Builder b(tri_box, cen);
-        b.order = tris;
-        b.nodes.reserve(2 * tris.size());
-        const int root = b.build(0, (int)tris.size());
+        built.emplace_back(Builder(tri_box, cen), 0);
+        built.back().first.order = tris;
+        built.back().first.nodes.reserve(2 * tris.size());
+    }
+    run_parallel(built.size(), [&](size_t g) {
+        Builder &b = built[g].first;
+        built[g].second = b.build(0, (int)b.order.size());
+    });
+    size_t gi = 0;
+    for (auto &[sid, tris] : groups) {
+        const Builder &b = built[gi].first;
+        const int root = built[gi++].second;
         const int off = (int)all.size(), base = (int)order_all.size();
         for (Node n : b.nodes) {
             if (n.count > 0) {

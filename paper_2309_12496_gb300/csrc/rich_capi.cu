@@ -15,6 +15,7 @@
 
 #include "rich_bvh.h"
 #include "rich_internal.h"
+#include "rich_proxy.h"
 
 using namespace rich;
 
@@ -109,8 +110,8 @@ struct rich_ctx {
     // refinement side records, one per storable hit
     RefineRec *d_refine = nullptr;
     uint64_t refine_cap = 0;
-    // occupancy per (external, refine, threads, smem), queried once
-    std::map<std::tuple<bool, bool, int, int, size_t>, int> occupancy;
+    // occupancy per (external, refine, proxies, class, threads, smem), queried once
+    std::map<std::tuple<bool, bool, bool, int, int, size_t>, int> occupancy;
     int smem_optin = 48 * 1024;
     // gradient: nominal tiles (host), their frames (device), tilted copies
     std::vector<rich_sphere> nom_spheres;
@@ -428,6 +429,15 @@ rich_status emit_core(rich_ctx *ctx, const rich_tracks *t, uint64_t seed, float 
     return RICH_OK;
 }
 
+// BVH nodes staged in shared memory by a trace block: the option's value, or
+// by default 256 in the wide blocks; with surface proxies few rays reach the
+// BVH, and 16 nodes leave the L1 to the cells and triangles.
+int staged_nodes(const rich_ctx *ctx, int opt, int threads, bool proxies) {
+    if (ctx->sc.n_tris == 0) return 0;
+    const int n = opt >= 0 ? opt : (threads > 256 ? (proxies ? 16 : 256) : 0);
+    return std::min(n, (int)ctx->sc.n_nodes);
+}
+
 // Azimuth order of the photons of the last emission. The buffer is sized
 // from the largest photon total the host has read (with a margin); an
 // emission that does not fit is traced in index order (device flag).
@@ -664,7 +674,11 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
     for (int64_t i = 0; i < nt; ++i)
         if (g->tri_material[i] < 0 || g->tri_material[i] >= g->n_materials)
             return bad("triangle material index");
-    if (!build_bvh(g->tri_vertices, g->tri_surface, nt, bvh, berr)) return bad(berr);
+    try {
+        if (!build_bvh(g->tri_vertices, g->tri_surface, nt, bvh, berr)) return bad(berr);
+    } catch (const std::exception &e) {      // the host builders allocate
+        return fail(ctx, RICH_ERR_OOM, std::string("rich_init_geometry: BVH: ") + e.what());
+    }
     if (bvh.depth >= RICH_BVH_STACK) return bad("BVH deeper than the traversal stack");
     // structural check: children point strictly forward (traversal ends),
     // leaf ranges stay inside the triangle array
@@ -718,6 +732,23 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
         split(d11, Q.d11);
         split(den != 0.0 ? 1.0 / den : 0.0, Q.inv_den);
     }
+    // ---- surface proxies of the meshes (none: the trace walks the BVH)
+    ProxyResult proxy;
+    {
+        double extent = 0.0;
+        for (const DevTri &T : tris)
+            for (float x : {T.v0x, T.v0y, T.v0z, T.v1x, T.v1y, T.v1z, T.v2x, T.v2y, T.v2z})
+                extent = std::max(extent, (double)std::fabs(x));
+        for (const DevRect &R : rects) {
+            for (float x : {R.ox, R.oy, R.oz})
+                extent = std::max(extent, (double)std::fabs(x) + std::max(R.w, R.h));
+        }
+        try {
+            build_proxies(tris, extent, proxy);
+        } catch (const std::exception &e) {
+            return fail(ctx, RICH_ERR_OOM, std::string("rich_init_geometry: proxies: ") + e.what());
+        }
+    }
     std::vector<DevTable> tables(g->n_tables);
     for (int i = 0; i < g->n_tables; ++i) std::memcpy(&tables[i], &g->tables[i], sizeof(DevTable));
     std::vector<DevMaterial> mats(g->n_materials);
@@ -728,11 +759,16 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
     size_t sizes[] = {sizeof(DevSphereGroup) * groups.size(), sizeof(DevTile) * tiles.size(),
                       sizeof(DevRect) * rects.size(), sizeof(DevTable) * tables.size(), sizeof(DevMaterial) * mats.size(),
                       sizeof(DevNode) * bvh.nodes.size(), sizeof(DevTri) * tris.size(),
-                      sizeof(float) * normals.size(), sizeof(DevTriRef) * tri_ref.size()};
+                      sizeof(float) * normals.size(), sizeof(DevTriRef) * tri_ref.size(),
+                      sizeof(DevProxy) * proxy.proxies.size(),
+                      sizeof(DevProxyCell) * proxy.cells.size(),
+                      sizeof(int32_t) * proxy.lists.size()};
     const void *srcs[] = {groups.data(), tiles.data(), rects.data(), tables.data(), mats.data(), bvh.nodes.data(), tris.data(),
-                          normals.data(), tri_ref.data()};
-    size_t total = 0, offs[9];
-    for (int i = 0; i < 9; ++i) {
+                          normals.data(), tri_ref.data(), proxy.proxies.data(),
+                          proxy.cells.data(), proxy.lists.data()};
+    constexpr int kArrays = (int)(sizeof sizes / sizeof sizes[0]);
+    size_t total = 0, offs[kArrays];
+    for (int i = 0; i < kArrays; ++i) {
         offs[i] = total;
         total += r256(sizes[i]);
     }
@@ -744,7 +780,7 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
     void *buf = nullptr;
     RICH_CUDA(cudaMalloc(&buf, std::max<size_t>(total, 256)));
     ctx->d_geom = buf;
-    for (int i = 0; i < 9; ++i)
+    for (int i = 0; i < kArrays; ++i)
         if (sizes[i]) RICH_CUDA(cudaMemcpy((char *)buf + offs[i], srcs[i], sizes[i], cudaMemcpyHostToDevice));
     SceneView sc{};
     auto at = [&](int i) { return sizes[i] ? (const void *)((char *)buf + offs[i]) : nullptr; };
@@ -757,6 +793,10 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
     sc.tris = (const DevTri *)at(6);
     sc.tri_normals = (const float *)at(7);
     sc.tri_ref = (const DevTriRef *)at(8);
+    sc.proxies = (const DevProxy *)at(9);
+    sc.proxy_cells = (const DevProxyCell *)at(10);
+    sc.proxy_lists = (const int32_t *)at(11);
+    sc.n_proxies = (int)proxy.proxies.size();
     sc.n_groups = (int)groups.size();
     sc.n_tiles = (int)tiles.size();
     sc.n_rects = (int)rects.size();
@@ -935,10 +975,7 @@ static rich_status trace_impl(rich_ctx *ctx, const rich_photons *in, const rich_
         return fail(ctx, RICH_ERR_STATE,
                     "rich_trace: the emission's spectrum table is not in the current scene");
     const int cls = trace_shape_class(threads, o->wide_regs != 0);
-    int smem_nodes = o->bvh_smem_nodes;
-    if (smem_nodes < 0) smem_nodes = threads > 256 ? 256 : 0;
-    if (smem_nodes > ctx->sc.n_nodes) smem_nodes = ctx->sc.n_nodes;
-    if (ctx->sc.n_tris == 0) smem_nodes = 0;
+    const int smem_nodes = staged_nodes(ctx, o->bvh_smem_nodes, threads, ctx->sc.n_proxies > 0 && !work);
     DeviceGuard guard(ctx->device);
     const bool refine = o->precision == RICH_PREC_REFINE64;
     const uint64_t hit_cap = out->hits ? out->hit_capacity : 0;
@@ -983,11 +1020,12 @@ static rich_status trace_impl(rich_ctx *ctx, const rich_photons *in, const rich_
         return fail(ctx, RICH_ERR_ARG, "rich_trace: staged BVH nodes exceed shared memory");
     int bps = o->blocks_per_sm;
     {
-        const auto key = std::make_tuple(in != nullptr, refine, cls, threads, shape.smem);
+        const bool proxy = ctx->sc.n_proxies > 0 && !work;
+        const auto key = std::make_tuple(in != nullptr, refine, proxy, cls, threads, shape.smem);
         auto it = ctx->occupancy.find(key);
         if (it == ctx->occupancy.end())
             it = ctx->occupancy.emplace(key, trace_blocks_per_sm(in != nullptr, refine, cls,
-                                                                 threads, shape.smem)).first;
+                                                                 threads, shape.smem, proxy)).first;
         if (it->second < 1)
             return fail(ctx, RICH_ERR_ARG, "rich_trace: launch shape does not fit on an SM");
         if (!bps || bps > it->second) bps = it->second;
@@ -1228,10 +1266,7 @@ RICH_API rich_status rich_trace_grad(rich_ctx *ctx, const rich_tracks *t,
     }
     const int threads = fo.block_threads ? fo.block_threads : kDefaultThreads;
     const int cls = trace_shape_class(threads, fo.wide_regs != 0);
-    int smem_nodes = fo.bvh_smem_nodes;
-    if (smem_nodes < 0) smem_nodes = threads > 256 ? 256 : 0;
-    if (smem_nodes > ctx->sc.n_nodes) smem_nodes = ctx->sc.n_nodes;
-    if (ctx->sc.n_tris == 0) smem_nodes = 0;
+    const int smem_nodes = staged_nodes(ctx, fo.bvh_smem_nodes, threads, sv.n_proxies > 0);
     TraceParams p{};
     p.precision = RICH_PREC_REFINE64;
     p.max_bounces = fo.max_bounces;
@@ -1256,7 +1291,8 @@ RICH_API rich_status rich_trace_grad(rich_ctx *ctx, const rich_tracks *t,
     shape.threads = threads;
     shape.cls = cls;
     shape.smem = trace_smem_bytes(sv, smem_nodes, threads, cls);
-    const int bps = trace_blocks_per_sm(false, true, cls, threads, shape.smem);
+    const int bps = trace_blocks_per_sm(false, true, cls, threads, shape.smem,
+                                        sv.n_proxies > 0);
     if (bps < 1) return fail(ctx, RICH_ERR_ARG, "rich_trace_grad: launch shape does not fit");
     shape.blocks = bps * ctx->n_sm;
     Counters *ctr = nullptr, *ctr_next = nullptr;

@@ -85,6 +85,35 @@ struct alignas(16) DevNode { // 128 B: boxes of up to four children (by axis) + 
     int32_t pad[4];
 };
 
+// One sphere (r > 0) or plane (r = 0) that a set of meshed surfaces follows,
+// and the grid over its projection along the axis (rich_proxy.h).
+#define RICH_MAX_PROXIES 8
+struct alignas(16) DevProxy {  // 128 B
+    float cx, cy, cz, r;       // centre and radius, or a point of the plane
+    float ax, ay, az, z_min;   // axis from the centre to the cap (normal of the plane);
+                               // lower bound of (p - c) . axis over the cap
+    float e1x, e1y, e1z, x0;   // grid axes and corner
+    float e2x, e2y, e2z, y0;
+    float inv_cell, fnx, fny;  // 1 / cell size, grid size
+    int32_t nx;
+    float r2, h2_min, q2_max;  // r^2, (r cos_min)^2, squared outer radius of the shell
+    float dt;                  // bound of the along-ray distance from crossing to facet
+    float w2_max;              // squared distance up to which the bounds hold
+    float gx, gy, gz;          // sphere bounding the mesh: centre - c, squared radius
+    float g2;
+    int32_t first_cell;
+    int32_t surf;              // BVH reference of its surface when it has exactly one,
+                               // else 0x7FFFFFFF
+    int32_t pad;
+};
+
+// Triangles (leaf positions) that a ray through the cell can meet: up to two
+// by themselves (-1: none), else a = first entry of a list and b = 0x80000000 |
+// its length.
+struct alignas(8) DevProxyCell {
+    int32_t a, b;
+};
+
 // Per triangle (leaf order), constants of the double-word refinement formed
 // once on the host in FP64 and stored as hi + lo pairs: the unit geometric
 // normal and, for the barycentrics of the smooth normal, the edge dot
@@ -126,7 +155,10 @@ struct SceneView {
     const DevTri *tris;
     const float *tri_normals;   // 9 floats per triangle, leaf order, or null
     const DevTriRef *tri_ref;   // per triangle, leaf order
-    int32_t n_groups, n_tiles, n_rects, n_tables, n_materials, n_nodes;
+    const DevProxy *proxies;    // surface proxies covering every triangle, or null
+    const DevProxyCell *proxy_cells;
+    const int32_t *proxy_lists;
+    int32_t n_groups, n_tiles, n_rects, n_tables, n_materials, n_nodes, n_proxies;
     int64_t n_tris;
     int32_t tri_prim_base;
     int32_t n_planes;
@@ -299,7 +331,7 @@ cudaError_t launch_adjoint(const SceneView &sc, const EmitView &em, const TraceP
                            cudaStream_t s);
 size_t trace_smem_bytes(const SceneView &sc, int smem_nodes, int threads, int cls);
 int trace_shape_class(int threads, bool wide);
-int trace_blocks_per_sm(bool ext, bool refine, int cls, int threads, size_t smem);
+int trace_blocks_per_sm(bool ext, bool refine, int cls, int threads, size_t smem, bool proxy);
 int yield_block_threads();
 
 }  // namespace rich
