@@ -964,10 +964,7 @@ __device__ __forceinline__ void nearest_rects(const SmemScene &S, f3 o, f3 d,
 struct Ray {
     f3 o, d, inv;
     float sx, sy, sz;
-    int k;              // axes of the watertight test: kx | ky << 2 | kz << 4
-    __device__ __forceinline__ int kx() const { return k & 3; }
-    __device__ __forceinline__ int ky() const { return (k >> 2) & 3; }
-    __device__ __forceinline__ int kz() const { return k >> 4; }
+    int kz;             // the direction's largest component
 };
 
 __device__ __forceinline__ float pick(float x, float y, float z, int k) {
@@ -984,36 +981,42 @@ __device__ __forceinline__ Ray make_ray(f3 o, f3 d) {
                 1.0f / (fabsf(d.z) > eps ? d.z : copysignf(eps, d.z)));
     const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
     int kz = (ax > ay) ? (ax > az ? 0 : 2) : (ay > az ? 1 : 2);
-    int kx = kz == 2 ? 0 : kz + 1;
-    int ky = kx == 2 ? 0 : kx + 1;
+    // (exchanging x and y for dz < 0, as the published test does to keep the
+    // winding, would negate the edge functions and their sum alone: both
+    // windings are accepted, so the quotients are the same)
     const float dz = pick(d.x, d.y, d.z, kz);
-    if (dz < 0.0f) {
-        int tmp = kx;
-        kx = ky;
-        ky = tmp;
-    }
-    r.k = kx | ky << 2 | kz << 4;
-    r.sx = pick(d.x, d.y, d.z, kx) / dz;
-    r.sy = pick(d.x, d.y, d.z, ky) / dz;
+    r.kz = kz;
+    r.sx = (kz == 2 ? d.x : (kz == 0 ? d.y : d.z)) / dz;
+    r.sy = (kz == 2 ? d.y : (kz == 0 ? d.z : d.x)) / dz;
     r.sz = 1.0f / dz;
     return r;
+}
+
+// (x, y, z) -> (y, z, x) for kz = 0, (z, x, y) for kz = 1
+__device__ __forceinline__ void rotate_axes(float &x, float &y, float &z, int kz) {
+    const float x0 = x, y0 = y, z0 = z;
+    x = kz == 0 ? y0 : z0;
+    y = kz == 0 ? z0 : x0;
+    z = kz == 0 ? x0 : y0;
 }
 
 __device__ __forceinline__ bool watertight(const Ray &r, const DevTri &T,
                                            float t_min, float t_max, float &t,
                                            float &b0, float &b1, float &b2) {
-    const float Ax0 = T.v0x - r.o.x, Ay0 = T.v0y - r.o.y, Az0 = T.v0z - r.o.z;
-    const float Bx0 = T.v1x - r.o.x, By0 = T.v1y - r.o.y, Bz0 = T.v1z - r.o.z;
-    const float Cx0 = T.v2x - r.o.x, Cy0 = T.v2y - r.o.y, Cz0 = T.v2z - r.o.z;
-    const int kx = r.kx(), ky = r.ky(), kz = r.kz();
-    const float Akz = pick(Ax0, Ay0, Az0, kz), Bkz = pick(Bx0, By0, Bz0, kz),
-                Ckz = pick(Cx0, Cy0, Cz0, kz);
-    const float Ax = fmaf(-r.sx, Akz, pick(Ax0, Ay0, Az0, kx));
-    const float Ay = fmaf(-r.sy, Akz, pick(Ax0, Ay0, Az0, ky));
-    const float Bx = fmaf(-r.sx, Bkz, pick(Bx0, By0, Bz0, kx));
-    const float By = fmaf(-r.sy, Bkz, pick(Bx0, By0, Bz0, ky));
-    const float Cx = fmaf(-r.sx, Ckz, pick(Cx0, Cy0, Cz0, kx));
-    const float Cy = fmaf(-r.sy, Ckz, pick(Cx0, Cy0, Cz0, ky));
+    float ax = T.v0x - r.o.x, ay = T.v0y - r.o.y, Akz = T.v0z - r.o.z;
+    float bx = T.v1x - r.o.x, by = T.v1y - r.o.y, Bkz = T.v1z - r.o.z;
+    float cx = T.v2x - r.o.x, cy = T.v2y - r.o.y, Ckz = T.v2z - r.o.z;
+    // turn the axes so that kz is the last; light that meets the mirrors
+    // mostly runs along z, so the warp passes this by (selects of each
+    // component instead: RICH1, 10^4 tracks, 653 -> 587 us without them)
+    if (r.kz != 2) {
+        rotate_axes(ax, ay, Akz, r.kz);
+        rotate_axes(bx, by, Bkz, r.kz);
+        rotate_axes(cx, cy, Ckz, r.kz);
+    }
+    const float Ax = fmaf(-r.sx, Akz, ax), Ay = fmaf(-r.sy, Akz, ay);
+    const float Bx = fmaf(-r.sx, Bkz, bx), By = fmaf(-r.sy, Bkz, by);
+    const float Cx = fmaf(-r.sx, Ckz, cx), Cy = fmaf(-r.sy, Ckz, cy);
     float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
     float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
