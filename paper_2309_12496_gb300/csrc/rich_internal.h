@@ -104,7 +104,8 @@ struct alignas(16) DevProxy {  // 128 B
     int32_t first_cell;
     int32_t surf;              // BVH reference of its surface when it has exactly one,
                                // else 0x7FFFFFFF
-    int32_t pad;
+    float t_far;               // a first estimate of a crossing below this is behind the
+                               // start (before its Newton step)
 };
 
 // Triangles (leaf positions) that a ray through the cell can meet: up to two

@@ -237,6 +237,9 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     const double out_r = f.r + f.shell + 2.0 * E + 4.0e-6 * W;
     P.q2_max = (float)(out_r * out_r);
     P.dt = (float)((f.shell + E) / kProxyCosMin + E);
+    // a direction that is unit to 1e-6 puts the first estimate off by at most
+    // 1e-6 t^2 / h, t <= 2 W and h >= r cos_min
+    P.t_far = (float)(-(double)P.dt - (sphere ? 4.0e-6 * W * W / (f.r * kProxyCosMin) : 0.0));
     P.w2_max = (float)(W * W);
     P.gx = (float)g[0]; P.gy = (float)g[1]; P.gz = (float)g[2];
     P.g2 = (float)((rho + E + 4.0e-6 * W) * (rho + E + 4.0e-6 * W));

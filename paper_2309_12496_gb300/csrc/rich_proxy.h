@@ -83,6 +83,7 @@ RICH_HD bool proxy_cells(const DevProxy &P, float ox, float oy, float oz, float 
     for (int k = 0; k < 2; ++k) {
         if (k >= n) continue;
         float tk = t[k];
+        if (tk < P.t_far) continue;      // behind the start whatever the roundings
         float px = fmaf(tk, dx, wx), py = fmaf(tk, dy, wy), pz = fmaf(tk, dz, wz);
         if (P.r > 0.0f) {
             // one Newton step on |p|^2 = r^2 (d|p|^2/dt = -+2h at the roots)
