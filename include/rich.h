@@ -287,8 +287,8 @@ typedef struct rich_trace_opts {
                                refractions), 1..RICH_MAX_BOUNCES             */
     int32_t max_steps;      /* surface interactions, 1..RICH_MAX_STEPS        */
     float t_min;            /* minimum hit distance after an interaction (mm) */
-    /* launch knobs (0 -> default: 512 threads of the 64-register build, two
-       blocks per SM, 256 staged top nodes) */
+    /* launch knobs (0 -> default: 1024 threads of the 64-register build, one
+       block per SM) */
     int32_t block_threads;  /* threads per block, multiple of 32, <= 1024;
                                above 256 the kernel is built for one block
                                per SM (see wide_regs); launched with 512
@@ -308,7 +308,8 @@ typedef struct rich_trace_opts {
                                walk does not use in shared memory          */
     int32_t bvh_smem_nodes; /* top BVH nodes (128 bytes each) staged in shared
                                memory per block by a TMA bulk copy
-                               (-1: default, 256 above 256 threads)         */
+                               (-1: default, above 256 threads 256, or 16
+                               when the meshes lie on surface proxies)       */
     /* Efficiencies applied before propagation (Sec. 4.3: the quantum
      * efficiency and the mirror reflectivities combined into one
      * accept/reject per photon at its wavelength, and rejected photons not

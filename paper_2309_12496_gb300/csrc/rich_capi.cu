@@ -22,10 +22,13 @@ using namespace rich;
 // A counter slot: a trace's counters and, right after them, the photon
 // total that trace saw, so one copy reads both.
 constexpr size_t kCtrBytes = sizeof(Counters) + sizeof(unsigned long long);
-// Default trace block: 512 threads of the 64-register build, two blocks per
-// SM (32 warps). Faster than one block of 1024 on the mesh and analytic
-// scenes alike (RICH1 -4 %, forward + adjoint -5 %).
-constexpr int kDefaultThreads = 512;
+// Default trace block: one of 1024 threads of the 64-register build per SM (32
+// warps), sharing one copy of the staged scene. Against two blocks of 512:
+// RICH1, 10^4 tracks, 579 -> 565 us, RICH2 4.92 -> 4.79 ms, 10^6 caller photons
+// 238 -> 231 us, analytic scenes equal. Fewer warps per SM are slower (28, 24 and
+// 20 of them: 620, 680, 763 us), and 40 or 48 warps at 48 or 40 registers spill
+// (682, 713 us).
+constexpr int kDefaultThreads = 1024;
 static_assert(sizeof(Counters) % 8 == 0, "the photon total follows the counters");
 
 // One step of rich_run_host / rich_run_host_async: where its counters land
@@ -797,6 +800,9 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
     sc.proxy_cells = (const DevProxyCell *)at(10);
     sc.proxy_lists = (const int32_t *)at(11);
     sc.n_proxies = (int)proxy.proxies.size();
+    sc.n_proxy_planes = proxy.n_planes;
+    sc.proxy_o2_max = proxy.o2_max;
+    sc.proxy_dt = proxy.dt_max;
     sc.n_groups = (int)groups.size();
     sc.n_tiles = (int)tiles.size();
     sc.n_rects = (int)rects.size();

@@ -85,27 +85,26 @@ struct alignas(16) DevNode { // 128 B: boxes of up to four children (by axis) + 
     int32_t pad[4];
 };
 
-// One sphere (r > 0) or plane (r = 0) that a set of meshed surfaces follows,
-// and the grid over its projection along the axis (rich_proxy.h).
+// One sphere or plane that a set of meshed surfaces follows, and the grid over
+// its projection along the axis, in units of its cells (rich_proxy.h).
 #define RICH_MAX_PROXIES 8
-struct alignas(16) DevProxy {  // 128 B
-    float cx, cy, cz, r;       // centre and radius, or a point of the plane
+struct alignas(16) DevProxy {  // 128 B, read as 16-byte words
+    float cx, cy, cz, dt;      // centre, or a point of the plane; bound of the along-ray
+                               // distance from crossing to facet
     float ax, ay, az, z_min;   // axis from the centre to the cap (normal of the plane);
                                // lower bound of (p - c) . axis over the cap
-    float e1x, e1y, e1z, x0;   // grid axes and corner
+    float e1x, e1y, e1z, x0;   // cell coordinates (p - c) . e1 - x0, (p - c) . e2 - y0
     float e2x, e2y, e2z, y0;
-    float inv_cell, fnx, fny;  // 1 / cell size, grid size
-    int32_t nx;
+    float fnx, fny;            // grid size
+    int32_t nx, first_cell;
     float r2, h2_min, q2_max;  // r^2, (r cos_min)^2, squared outer radius of the shell
-    float dt;                  // bound of the along-ray distance from crossing to facet
-    float w2_max;              // squared distance up to which the bounds hold
-    float gx, gy, gz;          // sphere bounding the mesh: centre - c, squared radius
-    float g2;
-    int32_t first_cell;
-    int32_t surf;              // BVH reference of its surface when it has exactly one,
-                               // else 0x7FFFFFFF
     float t_far;               // a first estimate of a crossing below this is behind the
                                // start (before its Newton step)
+    float gx, gy, gz, g2;      // sphere bounding the mesh: centre - c, squared radius
+    int32_t surf;              // BVH reference of its surface when it has exactly one,
+                               // else 0x7FFFFFFF
+    float r;                   // radius, 0 for a plane
+    int32_t pad[2];
 };
 
 // Triangles (leaf positions) that a ray through the cell can meet: up to two
@@ -160,6 +159,9 @@ struct SceneView {
     const DevProxyCell *proxy_cells;
     const int32_t *proxy_lists;
     int32_t n_groups, n_tiles, n_rects, n_tables, n_materials, n_nodes, n_proxies;
+    int32_t n_proxy_planes;     // the proxies' planes come first
+    float proxy_o2_max;         // |o|^2 up to which the proxies' bounds hold
+    float proxy_dt;             // largest DevProxy::dt
     int64_t n_tris;
     int32_t tri_prim_base;
     int32_t n_planes;

@@ -1284,24 +1284,74 @@ __device__ __noinline__ void nearest_bvh_far(const SceneView &sc, const DevNode 
 // instructions per RICH1 photon. Measured with the hits and fates the same:
 // trace of RICH1, 10^4 tracks, 1058 -> 725 us, of RICH2, 1.2 x 10^5 tracks,
 // 9.15 -> 6.01 ms, 10^6 caller photons on RICH1 463 -> 296 us a call.
+// Up to two crossings with cells are kept, nearest first (a third leaves the ray
+// to the BVH unless a nearer hit settles it), and their triangles are tested
+// after the last proxy, so that lanes whose mirrors differ test theirs together.
 template <bool EXT>
 __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemScene &S, f3 o, f3 d,
                                                 int skip, int skip_ref, float t_min, Best &b) {
-    // a caller's direction need not be a unit vector
+    // origins outside the scene's box, and callers' directions that are not
+    // unit vectors, are outside the proxies' bounds
+    if (!(dot3(o, o) <= sc.proxy_o2_max)) return false;
     if (EXT && !(fabsf(dot3(d, d) - 1.0f) <= 2.0e-6f)) return false;
-    const Ray r = make_ray(o, d);
-    bool all = true;
+    const float kInf = __int_as_float(0x7f800000);
+    float t0 = kInf, t1 = kInf, t2 = kInf;      // nearest three
+    int c0 = -1, c1 = -1;
+    auto keep = [&](float t, int c) {
+        t = c >= 0 ? t : kInf;
+        const bool l0 = t < t0, l1 = t < t1;
+        t2 = fminf(t2, l1 ? t1 : t);
+        c1 = l0 ? c0 : (l1 ? c : c1);
+        t1 = l0 ? t0 : (l1 ? t : t1);
+        c0 = l0 ? c : c0;
+        t0 = l0 ? t : t0;
+    };
+    unsigned unsure = 0, entering = 0;
+    int i = 0;
 #pragma unroll 1
-    for (int i = 0; i < S.n_proxies; ++i) {
+    for (; i < sc.n_proxy_planes; ++i) {
         const DevProxy &P = S.proxies()[i];
-        if (P.surf == skip_ref && skip_ref != kNoSurf) continue;
-        int cell[2];
-        all = proxy_cells(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, cell) && all;
+        float t;
+        bool sure;
+        const int c = proxy_plane(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure);
+        const bool own = P.surf == skip_ref && skip_ref != kNoSurf;
+        unsure |= (unsigned)(!sure & !own) << i;
+        keep(t, own ? -1 : c);
+    }
+#pragma unroll 1
+    for (; i < S.n_proxies; ++i) {
+        const DevProxy &P = S.proxies()[i];
+        float t, sb, h2;
+        bool sure, ent;
+        const int c = proxy_sphere(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure, ent, sb, h2);
+        const bool own = P.surf == skip_ref && skip_ref != kNoSurf;
+        unsure |= (unsigned)(!sure & !own) << i;
+        entering |= (unsigned)(ent & !own) << i;
+        keep(t, own ? -1 : c);
+    }
+    while (entering) {                   // mostly the sphere just left
+        const DevProxy &P = S.proxies()[__ffs(entering) - 1];
+        entering &= entering - 1u;
+        const float wx = o.x - P.cx, wy = o.y - P.cy, wz = o.z - P.cz;
+        const float sb = fmaf(wx, d.x, fmaf(wy, d.y, wz * d.z));
+        const float qx = fmaf(-sb, d.x, wx), qy = fmaf(-sb, d.y, wy), qz = fmaf(-sb, d.z, wz);
+        const float h2 = P.r2 - fmaf(qx, qx, fmaf(qy, qy, qz * qz));
+        float t;
+        const int c = proxy_sphere_side(P, wx, wy, wz, d.x, d.y, d.z, sb, h2, -1.0f, t_min, b.t, t,
+                                        true);
+        keep(t, c);
+    }
+    bool all = true;
+    while (unsure) {
+        const DevProxy &P = S.proxies()[__ffs(unsure) - 1];
+        unsure &= unsure - 1u;
+        all = proxy_misses(P, o.x, o.y, o.z, d.x, d.y, d.z) && all;
+    }
+    if (c0 >= 0) {
+        const Ray r = make_ray(o, d);
 #pragma unroll 1
         for (int k = 0; k < 2; ++k) {
-            if (k) cell[0] = cell[1];
-            if (cell[0] < 0) continue;
-            const int2 c = __ldg(reinterpret_cast<const int2 *>(sc.proxy_cells + cell[0]));
+            const int2 c = __ldg(reinterpret_cast<const int2 *>(sc.proxy_cells + c0));
             const bool list = c.y < -1;
             const int n = list ? (c.y & 0x7FFFFFFF) : (c.x >= 0) + (c.y >= 0);
 #pragma unroll 1
@@ -1311,7 +1361,10 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
                 if (T.prim == skip || (T.pad == skip_ref && skip_ref != kNoSurf)) continue;
                 test_tri(sc, r, T, tri, t_min, b);
             }
+            if (c1 < 0 || t1 > b.t + sc.proxy_dt) break;
+            c0 = c1;
         }
+        all = all && t2 > b.t + sc.proxy_dt;
     }
     return all;
 }

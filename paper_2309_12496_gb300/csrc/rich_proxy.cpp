@@ -56,6 +56,9 @@ struct Fit {
     std::vector<int> tris;
 };
 
+// Largest |o| of an origin in the scene's box [-extent, extent]^3.
+double o_max(double extent) { return 1.75 * extent; }
+
 V3 round32(const V3 &a) { return {(double)(float)a[0], (double)(float)a[1], (double)(float)a[2]}; }
 
 // Largest distance of the triangles from the sphere or plane: for a sphere
@@ -206,8 +209,9 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     double rho = 0.0;
     for (int i : f.tris)
         for (int v = 0; v < 3; ++v) rho = std::max(rho, len(sub(sub(vert(T[i], v), f.c), g)));
-    // distances from c up to which the bounds are to hold, and the margins
-    const double W = f.r + 2.0 * extent + 4.0 * rho;
+    // distances from c up to which the bounds are to hold (origins anywhere in
+    // the scene's box), and the margins
+    const double W = o_max(extent) + len(f.c);
     const double E = 32.0 * kUnit * W;
     const double margin = (f.shell + E) / kProxyCosMin + E;
     const double tri_size = std::sqrt(area / (double)f.tris.size());
@@ -218,29 +222,31 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     // long thin meshes: no more than `most` cells along either side
     size = std::max(size, std::max(wx, wy) / most);
     if (!(size > 0.0) || !(4.0 * margin <= tri_size)) return false;
-    const float inv = (float)(1.0 / size);
-    size = 1.0 / (double)inv;
-    const float x0 = (float)(lo[0] - 2.0 * margin), y0 = (float)(lo[1] - 2.0 * margin);
-    const int nx = (int)std::ceil((hi[0] + 2.0 * margin - x0) / size) + 1;
-    const int ny = (int)std::ceil((hi[1] + 2.0 * margin - y0) / size) + 1;
+    // cell coordinates: FP32 axes divided by the cell size (only their linear
+    // map matters) and FP32 corner
+    const V3 f1 = round32({e1[0] / size, e1[1] / size, e1[2] / size});
+    const V3 f2 = round32({e2[0] / size, e2[1] / size, e2[2] / size});
+    const double m = margin / size * (1.0 + 1.0e-6);
+    const float x0 = (float)(lo[0] / size - 2.0 * m), y0 = (float)(lo[1] / size - 2.0 * m);
+    const int nx = (int)std::ceil(hi[0] / size + 2.0 * m - x0) + 1;
+    const int ny = (int)std::ceil(hi[1] / size + 2.0 * m - y0) + 1;
     if ((double)nx * ny > 2.0e8) return false;
     DevProxy P;
     std::memset(&P, 0, sizeof P);
     P.cx = (float)f.c[0]; P.cy = (float)f.c[1]; P.cz = (float)f.c[2]; P.r = (float)f.r;
+    P.dt = (float)((f.shell + E) / kProxyCosMin + E);
     P.ax = (float)axis[0]; P.ay = (float)axis[1]; P.az = (float)axis[2];
     P.z_min = (float)(0.5 * lo[2]);
-    P.e1x = (float)e1[0]; P.e1y = (float)e1[1]; P.e1z = (float)e1[2]; P.x0 = x0;
-    P.e2x = (float)e2[0]; P.e2y = (float)e2[1]; P.e2z = (float)e2[2]; P.y0 = y0;
-    P.inv_cell = inv; P.fnx = (float)nx; P.fny = (float)ny; P.nx = nx;
+    P.e1x = (float)f1[0]; P.e1y = (float)f1[1]; P.e1z = (float)f1[2]; P.x0 = x0;
+    P.e2x = (float)f2[0]; P.e2y = (float)f2[1]; P.e2z = (float)f2[2]; P.y0 = y0;
+    P.fnx = (float)nx; P.fny = (float)ny; P.nx = nx;
     P.r2 = (float)(f.r * f.r);
     P.h2_min = (float)(f.r * f.r * kProxyCosMin * kProxyCosMin);
     const double out_r = f.r + f.shell + 2.0 * E + 4.0e-6 * W;
     P.q2_max = (float)(out_r * out_r);
-    P.dt = (float)((f.shell + E) / kProxyCosMin + E);
     // a direction that is unit to 1e-6 puts the first estimate off by at most
     // 1e-6 t^2 / h, t <= 2 W and h >= r cos_min
     P.t_far = (float)(-(double)P.dt - (sphere ? 4.0e-6 * W * W / (f.r * kProxyCosMin) : 0.0));
-    P.w2_max = (float)(W * W);
     P.gx = (float)g[0]; P.gy = (float)g[1]; P.gz = (float)g[2];
     P.g2 = (float)((rho + E + 4.0e-6 * W) * (rho + E + 4.0e-6 * W));
     P.surf = T[f.tris[0]].pad;
@@ -254,24 +260,24 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
         double q[3][2], blo[2] = {HUGE_VAL, HUGE_VAL}, bhi[2] = {-HUGE_VAL, -HUGE_VAL};
         for (int v = 0; v < 3; ++v) {
             const V3 w = sub(vert(T[i], v), f.c);
-            q[v][0] = dot(w, e1) - (double)x0;
-            q[v][1] = dot(w, e2) - (double)y0;
+            q[v][0] = dot(w, f1) - (double)x0;
+            q[v][1] = dot(w, f2) - (double)y0;
             for (int k = 0; k < 2; ++k) {
-                blo[k] = std::min(blo[k], q[v][k] - margin);
-                bhi[k] = std::max(bhi[k], q[v][k] + margin);
+                blo[k] = std::min(blo[k], q[v][k] - m);
+                bhi[k] = std::max(bhi[k], q[v][k] + m);
             }
         }
         const double turn = (q[1][0] - q[0][0]) * (q[2][1] - q[0][1]) -
                             (q[1][1] - q[0][1]) * (q[2][0] - q[0][0]);
         const double sg = turn < 0.0 ? -1.0 : 1.0;
-        const int ix0 = std::max(0, (int)std::floor(blo[0] / size));
-        const int iy0 = std::max(0, (int)std::floor(blo[1] / size));
-        const int ix1 = std::min(nx - 1, (int)std::floor(bhi[0] / size));
-        const int iy1 = std::min(ny - 1, (int)std::floor(bhi[1] / size));
-        const double half = 0.5 * size + margin;
+        const int ix0 = std::max(0, (int)std::floor(blo[0]));
+        const int iy0 = std::max(0, (int)std::floor(blo[1]));
+        const int ix1 = std::min(nx - 1, (int)std::floor(bhi[0]));
+        const int iy1 = std::min(ny - 1, (int)std::floor(bhi[1]));
+        const double half = 0.5 + m;
         for (int iy = iy0; iy <= iy1; ++iy)
             for (int ix = ix0; ix <= ix1; ++ix) {
-                const double mx = (ix + 0.5) * size, my = (iy + 0.5) * size;
+                const double mx = ix + 0.5, my = iy + 0.5;
                 bool apart = false;
                 for (int v = 0; v < 3 && !apart; ++v) {
                     const double *a = q[v], *b = q[(v + 1) % 3];
@@ -350,6 +356,8 @@ void build_proxies(const std::vector<DevTri> &T, double extent, ProxyResult &out
         }
         home->tris.insert(home->tris.end(), order[i]->begin(), order[i]->end());
     }
+    std::stable_sort(fits.begin(), fits.end(),
+                     [](const Fit &a, const Fit &b) { return a.r == 0.0 && b.r > 0.0; });
     // all surfaces of a fit together, then its grid
     std::vector<ProxyResult> part(fits.size());
     run_parallel(fits.size(), [&](size_t k) {
@@ -369,7 +377,10 @@ void build_proxies(const std::vector<DevTri> &T, double extent, ProxyResult &out
             out.cells.push_back(c);
         }
         out.lists.insert(out.lists.end(), p.lists.begin(), p.lists.end());
+        out.n_planes += p.proxies[0].r == 0.0f;
+        out.dt_max = std::max(out.dt_max, p.proxies[0].dt);
     }
+    out.o2_max = (float)(o_max(extent) * o_max(extent));
 }
 
 }  // namespace rich

@@ -27,81 +27,94 @@
 
 namespace rich {
 
-// One proxy against a ray: cell[k] >= 0 is the cell to test at the ray's
-// k-th crossing (two for a sphere, nearer first), -1 none. Returns false when
-// the ray may meet the mesh but the margin does not hold (take the BVH).
-// t_max: the nearest hit known so far; (dx, dy, dz) a unit vector to 1e-6.
+// The crossings of one ray with one proxy. cell >= 0: the cell to look up at
+// distance t; -1: the ray cannot meet the mesh there. sure: the margins hold
+// for this ray; if not, proxy_misses says whether the ray passes the mesh by
+// (else the BVH has to take it). t_max: the nearest hit known so far;
+// (dx, dy, dz) a unit vector to 1e-6, |o| at most the scene's o_max.
 //
-// The bounds: with u = 2^-24 and W = sqrt(w2_max) >= |o - c|, the FP32
-// crossing point differs from the ray's exact crossing of the sphere or
-// plane by at most 8 u W across the surface (the roundings of w, of the
-// dots and, after the Newton step on |p| = r, of |p|^2 - r^2), by 8 u W / c
-// along the ray for an angle of incidence with cosine c >= kProxyCosMin,
-// and a facet's point lies within `shell` of the surface; the cells' margin
-// holds (shell + E) / kProxyCosMin + E with E = 32 u W.
+// The bounds: with u = 2^-24 and W >= |o - c|, the FP32 crossing point differs
+// from the ray's exact crossing of the sphere or plane by at most 8 u W across
+// the surface (the roundings of w, of the dots and, after the Newton step on
+// |p| = r, of |p|^2 - r^2), by 8 u W / c along the ray for an angle of
+// incidence with cosine c >= kProxyCosMin, and a facet's point lies within
+// `shell` of the surface; the cells' margin holds (shell + E) / kProxyCosMin + E
+// with E = 32 u W. The functions select instead of branching: a warp's rays
+// mostly take the same surfaces, and control flow was a fifth of the trace's
+// instructions.
 constexpr float kProxyCosMin = 0.25f;
 
-RICH_HD bool proxy_cells(const DevProxy &P, float ox, float oy, float oz, float dx, float dy,
-                         float dz, float t_min, float t_max, int cell[2]) {
-    cell[0] = cell[1] = -1;
-    const float wx = ox - P.cx, wy = oy - P.cy, wz = oz - P.cz;
-    const float w2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
-    bool sure = w2 <= P.w2_max;
-    const float b = fmaf(wx, dx, fmaf(wy, dy, wz * dz));
-    float t[2];
-    int n = 1;
-    float half_inv_h = 0.0f;
-    if (P.r > 0.0f) {
-        const float qx = fmaf(-b, dx, wx), qy = fmaf(-b, dy, wy), qz = fmaf(-b, dz, wz);
-        const float q2 = fmaf(qx, qx, fmaf(qy, qy, qz * qz));
-        if (sure && q2 > P.q2_max) return true;                  // passes outside the shell
-        const float h2 = P.r2 - q2;
-        sure = sure && h2 >= P.h2_min;
-        if (sure) {
-            const float h = sqrtf(h2);
-            half_inv_h = 0.5f / h;
-            t[0] = -b - h;
-            t[1] = -b + h;
-            n = 2;
-        }
-    } else {
-        const float den = fmaf(dx, P.ax, fmaf(dy, P.ay, dz * P.az));
-        sure = sure && fabsf(den) >= kProxyCosMin;
-        if (sure) t[0] = -fmaf(wx, P.ax, fmaf(wy, P.ay, wz * P.az)) / den;
-    }
-    if (!sure) {
-        // may the ray meet the sphere that bounds the mesh?
-        const float gx = wx - P.gx, gy = wy - P.gy, gz = wz - P.gz;
-        const float gb = fmaf(gx, dx, fmaf(gy, dy, gz * dz));
-        const float mx = fmaf(-gb, dx, gx), my = fmaf(-gb, dy, gy), mz = fmaf(-gb, dz, gz);
-        const float m2 = fmaf(mx, mx, fmaf(my, my, mz * mz));
-        return w2 <= P.w2_max && m2 > P.g2;
-    }
 #ifdef __CUDA_ARCH__
-#pragma unroll
+RICH_HD float proxy_div(float a, float b) { return __fdividef(a, b); }
+RICH_HD float proxy_rsqrt(float a) { return rsqrtf(a); }
+#else
+RICH_HD float proxy_div(float a, float b) { return a / b; }
+RICH_HD float proxy_rsqrt(float a) { return 1.0f / sqrtf(a); }
 #endif
-    for (int k = 0; k < 2; ++k) {
-        if (k >= n) continue;
-        float tk = t[k];
-        if (tk < P.t_far) continue;      // behind the start whatever the roundings
-        float px = fmaf(tk, dx, wx), py = fmaf(tk, dy, wy), pz = fmaf(tk, dz, wz);
-        if (P.r > 0.0f) {
-            // one Newton step on |p|^2 = r^2 (d|p|^2/dt = -+2h at the roots)
-            const float f = fmaf(px, px, fmaf(py, py, fmaf(pz, pz, -P.r2)));
-            const float s = k == 0 ? f * half_inv_h : -f * half_inv_h;
-            tk += s;
-            px = fmaf(s, dx, px);
-            py = fmaf(s, dy, py);
-            pz = fmaf(s, dz, pz);
-            if (!(fmaf(px, P.ax, fmaf(py, P.ay, pz * P.az)) >= P.z_min)) continue;
-        }
-        if (tk < t_min - P.dt || tk > t_max + P.dt) continue;
-        const float x = (fmaf(px, P.e1x, fmaf(py, P.e1y, pz * P.e1z)) - P.x0) * P.inv_cell;
-        const float y = (fmaf(px, P.e2x, fmaf(py, P.e2y, pz * P.e2z)) - P.y0) * P.inv_cell;
-        if (!(x >= 0.0f && x < P.fnx && y >= 0.0f && y < P.fny)) continue;
-        cell[k] = P.first_cell + (int)y * P.nx + (int)x;
-    }
-    return true;
+
+// The cell of the point p (relative to c) at distance t, or -1.
+RICH_HD int proxy_cell(const DevProxy &P, float px, float py, float pz, float t, float t_min,
+                       float t_max, bool ok) {
+    const float x = fmaf(px, P.e1x, fmaf(py, P.e1y, fmaf(pz, P.e1z, -P.x0)));
+    const float y = fmaf(px, P.e2x, fmaf(py, P.e2y, fmaf(pz, P.e2z, -P.y0)));
+    ok = ok & (x >= 0.0f) & (x < P.fnx) & (y >= 0.0f) & (y < P.fny) & (t >= t_min - P.dt) &
+         (t <= t_max + P.dt);
+    return ok ? P.first_cell + (int)y * P.nx + (int)x : -1;
+}
+
+RICH_HD int proxy_plane(const DevProxy &P, float ox, float oy, float oz, float dx, float dy,
+                        float dz, float t_min, float t_max, float &t, bool &sure) {
+    const float wx = ox - P.cx, wy = oy - P.cy, wz = oz - P.cz;
+    const float den = fmaf(dx, P.ax, fmaf(dy, P.ay, dz * P.az));
+    t = -proxy_div(fmaf(wx, P.ax, fmaf(wy, P.ay, wz * P.az)), den);
+    sure = fabsf(den) >= kProxyCosMin;
+    return proxy_cell(P, fmaf(t, dx, wx), fmaf(t, dy, wy), fmaf(t, dz, wz), t, t_min, t_max, sure);
+}
+
+// A sphere's crossing on leaving it (side = 1) or entering it (side = -1), from
+// b = w . d and h2 = r^2 - |w - b d|^2 >= h2_min.
+RICH_HD int proxy_sphere_side(const DevProxy &P, float wx, float wy, float wz, float dx, float dy,
+                              float dz, float b, float h2, float side, float t_min, float t_max,
+                              float &t, bool ok) {
+    const float ih = side * proxy_rsqrt(h2);
+    t = fmaf(h2, ih, -b);
+    float px = fmaf(t, dx, wx), py = fmaf(t, dy, wy), pz = fmaf(t, dz, wz);
+    // one Newton step on |p|^2 = r^2 (d|p|^2/dt = +-2 h at the crossings)
+    const float s = -0.5f * ih * fmaf(px, px, fmaf(py, py, fmaf(pz, pz, -P.r2)));
+    t += s;
+    px = fmaf(s, dx, px);
+    py = fmaf(s, dy, py);
+    pz = fmaf(s, dz, pz);
+    ok = ok & (fmaf(px, P.ax, fmaf(py, P.ay, pz * P.az)) >= P.z_min);
+    return proxy_cell(P, px, py, pz, t, t_min, t_max, ok);
+}
+
+// The sphere's crossing on leaving; entering: whether the crossing on entering
+// may lie ahead too (proxy_sphere_side with side = -1 then finds its cell).
+RICH_HD int proxy_sphere(const DevProxy &P, float ox, float oy, float oz, float dx, float dy,
+                         float dz, float t_min, float t_max, float &t, bool &sure, bool &entering,
+                         float &b, float &h2) {
+    const float wx = ox - P.cx, wy = oy - P.cy, wz = oz - P.cz;
+    b = fmaf(wx, dx, fmaf(wy, dy, wz * dz));
+    const float qx = fmaf(-b, dx, wx), qy = fmaf(-b, dy, wy), qz = fmaf(-b, dz, wz);
+    const float q2 = fmaf(qx, qx, fmaf(qy, qy, qz * qz));
+    h2 = P.r2 - q2;
+    const bool meets = h2 >= P.h2_min;
+    sure = meets | (q2 > P.q2_max);
+    h2 = meets ? h2 : P.h2_min;
+    // -b - h >= t_far (behind the start whatever the roundings if below)
+    const float far = -b - P.t_far;
+    entering = meets & (far >= 0.0f) & (far * far >= h2);
+    return proxy_sphere_side(P, wx, wy, wz, dx, dy, dz, b, h2, 1.0f, t_min, t_max, t, meets);
+}
+
+// Whether the ray passes by the sphere that bounds the proxy's mesh.
+RICH_HD bool proxy_misses(const DevProxy &P, float ox, float oy, float oz, float dx, float dy,
+                          float dz) {
+    const float gx = ox - P.cx - P.gx, gy = oy - P.cy - P.gy, gz = oz - P.cz - P.gz;
+    const float gb = fmaf(gx, dx, fmaf(gy, dy, gz * dz));
+    const float mx = fmaf(-gb, dx, gx), my = fmaf(-gb, dy, gy), mz = fmaf(-gb, dz, gz);
+    return fmaf(mx, mx, fmaf(my, my, mz * mz)) > P.g2;
 }
 
 // Host builder. On return `proxies` is empty when some triangle fits no
@@ -110,6 +123,9 @@ struct ProxyResult {
     std::vector<DevProxy> proxies;
     std::vector<DevProxyCell> cells;
     std::vector<int32_t> lists;       // triangle lists of the cells with more than two
+    int n_planes = 0;                 // planes first, then spheres
+    float o2_max = 0.0f;              // |o|^2 up to which the bounds hold
+    float dt_max = 0.0f;              // largest dt of any proxy
 };
 
 // tris: in leaf order, DevTri::pad naming the triangle's surface; extent:

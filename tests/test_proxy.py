@@ -41,11 +41,26 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
     double tests = 0;
     for (int64_t i = 0; i < nr; ++i) {
         out[i] = 0;
-        for (const DevProxy &P : R.proxies) {
-            int cell[2];
-            if (!proxy_cells(P, o[3 * i], o[3 * i + 1], o[3 * i + 2], d[3 * i], d[3 * i + 1],
-                             d[3 * i + 2], 1e-3f, t_max, cell))
-                out[i] |= 2;
+        const float *O = o + 3 * i, *D = d + 3 * i;
+        if (!(O[0] * O[0] + O[1] * O[1] + O[2] * O[2] <= R.o2_max)) {
+            out[i] = 2;
+            continue;
+        }
+        for (size_t k = 0; k < R.proxies.size(); ++k) {
+            const DevProxy &P = R.proxies[k];
+            int cell[2] = {-1, -1};
+            float t, b2, h2;
+            bool sure, entering = false;
+            if ((int)k < R.n_planes) {
+                cell[0] = proxy_plane(P, O[0], O[1], O[2], D[0], D[1], D[2], 1e-3f, t_max, t, sure);
+            } else {
+                cell[0] = proxy_sphere(P, O[0], O[1], O[2], D[0], D[1], D[2], 1e-3f, t_max, t, sure,
+                                       entering, b2, h2);
+                if (entering)
+                    cell[1] = proxy_sphere_side(P, O[0] - P.cx, O[1] - P.cy, O[2] - P.cz, D[0], D[1],
+                                                D[2], b2, h2, -1.0f, 1e-3f, t_max, t, true);
+            }
+            if (!sure && !proxy_misses(P, O[0], O[1], O[2], D[0], D[1], D[2])) out[i] |= 2;
             for (int c : cell) {
                 if (c < 0) continue;
                 const DevProxyCell &L = R.cells[(size_t)c];
