@@ -704,6 +704,17 @@ struct Photon {
     int skip_ref;          // BVH subtree of the surface just left, or kNoSurf
 };
 
+// philox10 out of line, for the draw blocks that few photons need. A fifth of
+// the trace's stalls are instruction fetch: the code of its loop, run by 32
+// warps at different places, is larger than the caches near the schedulers, so
+// the rare paths (these draws, the dispersive wavelength, the track search, the
+// event sums of unrecorded hits) are calls, and loops over surfaces are not
+// unrolled (RICH1, 10^4 tracks, 565 -> 518 us; RICH2 4.37 -> 3.99 ms).
+__device__ __noinline__ u4 philox10_far(uint32_t c0, uint32_t c1, uint32_t c2, uint32_t c3,
+                                        uint32_t k0, uint32_t k1) {
+    return philox10(c0, c1, c2, c3, k0, k1);
+}
+
 // Wavelength from a binned emission spectrum (CDF table): the bin k with
 // c_k <= u < c_{k+1}, linear inside it, each operation rounded in FP32.
 __device__ __forceinline__ float spectrum_lambda(const DevTable &T, float u) {
@@ -718,7 +729,7 @@ __device__ __forceinline__ float spectrum_lambda(const DevTable &T, float u) {
 // sin^2 theta(lambda) / sin^2 theta(lambda_min); trial 0 takes block 0 word
 // 2 and block 3 word 3, trial t >= 1 block 8 + (t-1)/2; the last of 64
 // candidates stands.
-__device__ float disp_lambda(const TrackRec &tr, uint32_t j, const EmitView &em, uint32_t wl0,
+__device__ __noinline__ float disp_lambda(const TrackRec &tr, uint32_t j, const EmitView &em, uint32_t wl0,
                              uint32_t wa0) {
     const float il0 = __fdiv_rn(1.0f, em.disp_lambda0);
     const float omb = tr.tan_theta;
@@ -748,7 +759,7 @@ __device__ __forceinline__ float photon_wavelength(const TrackRec &tr, uint32_t 
                                                    const DevTable *spec) {
     if (spec) return spectrum_lambda(*spec, u24f(w0.z));
     if (em.dispersion) {
-        const u4 w3 = philox10(3u, j, tr.id, tr.event, em.key0, em.key1);
+        const u4 w3 = philox10_far(3u, j, tr.id, tr.event, em.key0, em.key1);
         return disp_lambda(tr, j, em, w0.z, w3.w);
     }
     return emit_lambda(u24f(w0.z), em.inv1, em.span);
@@ -782,7 +793,7 @@ __device__ __forceinline__ void emit_photon(const TrackRec &tr, uint32_t j,
     float sp, cp;
     sincospif(2.0f * u24f(w0.y), &sp, &cp);
     if (em.source == RICH_SOURCE_ISOTROPIC) {
-        const u4 w3 = philox10(3u, j, tr.id, tr.event, em.key0, em.key1);
+        const u4 w3 = philox10_far(3u, j, tr.id, tr.event, em.key0, em.key1);
         const float ct = 1.0f - 2.0f * u24f(w3.z);      // exact
         const float st = sqrtf(fmaxf(0.0f, (1.0f - ct) * (1.0f + ct)));
         ph.d = normalize3(mk3(st * cp, st * sp, ct));
@@ -936,6 +947,7 @@ __device__ __noinline__ f3 sphere_normal(const DevSphereGroup &G, f3 o, f3 d, fl
 
 __device__ __forceinline__ void nearest_rects(const SmemScene &S, f3 o, f3 d,
                                               int skip, float t_min, Best &b) {
+#pragma unroll 1
     for (int k = 0; k < S.n_rects; ++k) {
         const DevRect &R = S.rects()[k];
         if (R.prim == skip) continue;
@@ -1020,7 +1032,7 @@ __device__ __forceinline__ bool watertight(const Ray &r, const DevTri &T,
     float U = __fsub_rn(__fmul_rn(Cx, By), __fmul_rn(Cy, Bx));
     float V = __fsub_rn(__fmul_rn(Ax, Cy), __fmul_rn(Ay, Cx));
     float W = __fsub_rn(__fmul_rn(Bx, Ay), __fmul_rn(By, Ax));
-    if (U == 0.0f || V == 0.0f || W == 0.0f) {
+    if (__builtin_expect(U == 0.0f || V == 0.0f || W == 0.0f, 0)) {
         U = (float)((double)Cx * By - (double)Cy * Bx);
         V = (float)((double)Ax * Cy - (double)Ay * Cx);
         W = (float)((double)Bx * Ay - (double)By * Ax);
@@ -1657,6 +1669,12 @@ __device__ __forceinline__ void add_event_sums(const SceneView &sc, const TraceP
     }
 }
 
+__device__ __noinline__ void add_event_sums_far(const SceneView &sc, const TraceParams &P, bool on,
+                                                uint32_t event, int plane, float u, float v,
+                                                float lam, double *s_es) {
+    add_event_sums(sc, P, on, event, plane, ffv(u), ffv(v), lam, s_es);
+}
+
 // Efficiencies applied before propagation (Sec. 4.3): the FP32 product,
 // left to right, of the listed response tables at the photon's wavelength.
 __device__ __forceinline__ float prefilter_prob(const SmemScene &S, const TraceParams &P,
@@ -1680,7 +1698,7 @@ struct TraceArgs {
 __device__ __forceinline__ uint32_t refl_word(const Photon &ph, int k,
                                               const EmitView &em) {
     if (k < 4) return k == 0 ? ph.wr0 : (k == 1 ? ph.wr1 : (k == 2 ? ph.wr2 : ph.wr3));
-    u4 w = philox10(2u, ph.j, ph.id, ph.event, em.key0, em.key1);
+    u4 w = philox10_far(2u, ph.j, ph.id, ph.event, em.key0, em.key1);
     k -= 4;
     return k == 0 ? w.x : (k == 1 ? w.y : (k == 2 ? w.z : w.w));
 }
@@ -1704,13 +1722,29 @@ struct ColdState {
 __device__ __forceinline__ uint32_t cold_refl_word(const ColdState &c, int k,
                                                    const EmitView &em) {
     if (k < 4) return c.at(kCWr0 + k);
-    u4 w = philox10(2u, c.at(kCJ), c.at(kCId), c.at(kCEvent), em.key0, em.key1);
+    u4 w = philox10_far(2u, c.at(kCJ), c.at(kCId), c.at(kCEvent), em.key0, em.key1);
     k -= 4;
     return k == 0 ? w.x : (k == 1 ? w.y : (k == 2 ? w.z : w.w));
 }
 
 // PROXY: the scene's triangles all lie on surface proxies (the counting build
 // always walks the BVH: its tallies are the walk's).
+// Track holding photon g: 32-ary search of the offsets by a converged warp.
+__device__ __noinline__ int64_t find_track(const EmitView &em, uint64_t g, int lane) {
+    int64_t lo = 0, hi = em.n_tracks;
+    while (hi - lo > 32) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t idx = lo + lane * step;
+        const bool ok = idx < hi && em.offsets[idx] <= g;
+        const int L = 31 - __clz(__ballot_sync(kFull, ok));
+        lo = lo + L * step;
+        hi = (lo + step < hi) ? lo + step : hi;
+    }
+    const int64_t idx = lo + lane;
+    const bool ok = idx < hi && em.offsets[idx] <= g;
+    return lo + (31 - __clz(__ballot_sync(kFull, ok)));
+}
+
 template <bool EXT, bool REFINE, int THREADS, int MINB, bool PROXY, bool COUNT = false>
 __global__ void __launch_bounds__(THREADS, MINB)
 k_trace(TraceArgs A) {
@@ -1922,21 +1956,7 @@ k_trace(TraceArgs A) {
                     entry_track = (int64_t)e.y;
                 }
                 if (!EXT && pool_track < 0 && __any_sync(kFull, take && !from_entry)) {
-                    // 32-ary search for the track containing pool_next
-                    int64_t lo = 0, hi = em.n_tracks;
-                    while (hi - lo > 32) {
-                        const int64_t step = (hi - lo + 31) / 32;
-                        const int64_t idx = lo + lane * step;
-                        const bool ok = idx < hi && em.offsets[idx] <= pool_next;
-                        const unsigned m = __ballot_sync(kFull, ok);
-                        const int L = 31 - __clz(m);
-                        lo = lo + L * step;
-                        hi = (lo + step < hi) ? lo + step : hi;
-                    }
-                    const int64_t idx = lo + lane;
-                    const bool ok = idx < hi && em.offsets[idx] <= pool_next;
-                    const unsigned m = __ballot_sync(kFull, ok);
-                    pool_track = lo + (31 - __clz(m));
+                    pool_track = find_track(em, pool_next, lane);
                 }
                 int64_t my_track = from_entry ? entry_track : pool_track;
                 bool rejected = false;
@@ -2221,8 +2241,15 @@ k_trace(TraceArgs A) {
                 if (binned_here) bin_hit(sc, P, PH_EVENT, hplane, ix, iy);
             }
         }
-        add_event_sums(sc, P, binned_here, alive ? PH_EVENT : 0u, hplane, ffv(hu), ffv(hv),
-                       alive ? PH_LAM : 0.0f, s_es);
+        if constexpr (REFINE) {
+            // only hits beyond the record buffer
+            if (__any_sync(kFull, binned_here))
+                add_event_sums_far(sc, P, binned_here, alive ? PH_EVENT : 0u, hplane, hu, hv,
+                                   alive ? PH_LAM : 0.0f, s_es);
+        } else {
+            add_event_sums(sc, P, binned_here, alive ? PH_EVENT : 0u, hplane, ffv(hu), ffv(hv),
+                           alive ? PH_LAM : 0.0f, s_es);
+        }
         if (fate != 0) {
             const uint64_t g_fate = PH_G;
             if (g_fate < P.fate_capacity) P.fate[g_fate] = (uint8_t)fate;
