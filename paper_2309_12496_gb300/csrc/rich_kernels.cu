@@ -729,7 +729,7 @@ __device__ __forceinline__ float spectrum_lambda(const DevTable &T, float u) {
 // sin^2 theta(lambda) / sin^2 theta(lambda_min); trial 0 takes block 0 word
 // 2 and block 3 word 3, trial t >= 1 block 8 + (t-1)/2; the last of 64
 // candidates stands.
-__device__ __noinline__ float disp_lambda(const TrackRec &tr, uint32_t j, const EmitView &em, uint32_t wl0,
+__device__ float disp_lambda(const TrackRec &tr, uint32_t j, const EmitView &em, uint32_t wl0,
                              uint32_t wa0) {
     const float il0 = __fdiv_rn(1.0f, em.disp_lambda0);
     const float omb = tr.tan_theta;
@@ -751,16 +751,27 @@ __device__ __noinline__ float disp_lambda(const TrackRec &tr, uint32_t j, const 
     return lam;
 }
 
+__device__ __noinline__ float disp_lambda_far(const TrackRec &tr, uint32_t j, const EmitView &em,
+                                              uint32_t wl0, uint32_t wa0) {
+    return disp_lambda(tr, j, em, wl0, wa0);
+}
+
 // Wavelength of a fused-emission photon from its draws: the source's binned
 // spectrum, the dispersive radiator's law, or the Frank-Tamm 1/lambda^2 law
 // on the emission band.
+// FAR: the rare sources out of line (the trace; k_materialize runs one source
+// over all its photons).
+template <bool FAR>
 __device__ __forceinline__ float photon_wavelength(const TrackRec &tr, uint32_t j,
                                                    const EmitView &em, const u4 &w0,
                                                    const DevTable *spec) {
     if (spec) return spectrum_lambda(*spec, u24f(w0.z));
     if (em.dispersion) {
-        const u4 w3 = philox10_far(3u, j, tr.id, tr.event, em.key0, em.key1);
-        return disp_lambda(tr, j, em, w0.z, w3.w);
+        if (FAR)
+            return disp_lambda_far(
+                tr, j, em, w0.z, philox10_far(3u, j, tr.id, tr.event, em.key0, em.key1).w);
+        return disp_lambda(tr, j, em, w0.z,
+                           philox10(3u, j, tr.id, tr.event, em.key0, em.key1).w);
     }
     return emit_lambda(u24f(w0.z), em.inv1, em.span);
 }
@@ -783,6 +794,7 @@ __device__ __forceinline__ float disp_tan_f32(const EmitView &em, float omb, flo
 // a dispersive radiator takes tan(theta) of the photon's own wavelength.
 // Isotropic source (the scintillation light named in Sec. 6): the
 // direction is uniform on the sphere, cos(theta) = 1 - 2u from draw block 3.
+template <bool FAR>
 __device__ __forceinline__ void emit_photon(const TrackRec &tr, uint32_t j,
                                             const EmitView &em, const u4 &w0, float lam,
                                             Photon &ph) {
@@ -793,7 +805,8 @@ __device__ __forceinline__ void emit_photon(const TrackRec &tr, uint32_t j,
     float sp, cp;
     sincospif(2.0f * u24f(w0.y), &sp, &cp);
     if (em.source == RICH_SOURCE_ISOTROPIC) {
-        const u4 w3 = philox10_far(3u, j, tr.id, tr.event, em.key0, em.key1);
+        const u4 w3 = FAR ? philox10_far(3u, j, tr.id, tr.event, em.key0, em.key1)
+                          : philox10(3u, j, tr.id, tr.event, em.key0, em.key1);
         const float ct = 1.0f - 2.0f * u24f(w3.z);      // exact
         const float st = sqrtf(fmaxf(0.0f, (1.0f - ct) * (1.0f + ct)));
         ph.d = normalize3(mk3(st * cp, st * sp, ct));
@@ -828,7 +841,7 @@ __global__ void k_materialize(SceneView sc, EmitView em, uint64_t n, rich_photon
         Photon ph;
         const uint32_t j = (uint32_t)(g - em.offsets[lo]);
         const u4 w0 = philox10(0u, j, tr.id, tr.event, em.key0, em.key1);
-        emit_photon(tr, j, em, w0, photon_wavelength(tr, j, em, w0, spec), ph);
+        emit_photon<false>(tr, j, em, w0, photon_wavelength<false>(tr, j, em, w0, spec), ph);
         out.x[g] = ph.o.x;
         out.y[g] = ph.o.y;
         out.z[g] = ph.o.z;
@@ -1998,13 +2011,13 @@ k_trace(TraceArgs A) {
                         ph.g = toff + j;
                         const u4 w0 = philox10(0u, j, tr.id, tr.event, em.key0, em.key1);
                         const DevTable *spec = em.spectrum >= 0 ? S.tables() + em.spectrum : nullptr;
-                        const float lam = photon_wavelength(tr, j, em, w0, spec);
+                        const float lam = photon_wavelength<true>(tr, j, em, w0, spec);
                         // efficiencies before propagation (Sec. 4.3): only
                         // the wavelength is needed to decide
                         if (P.n_prefilter && !(u24f(w0.w) < prefilter_prob(S, P, lam)))
                             rejected = true;
                         else
-                            emit_photon(tr, j, em, w0, lam, ph);
+                            emit_photon<true>(tr, j, em, w0, lam, ph);
                     }
                     if (rejected) {
                         if (ph.g < P.fate_capacity) P.fate[ph.g] = (uint8_t)RICH_FATE_PREFILTERED;
