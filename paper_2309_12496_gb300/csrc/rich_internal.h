@@ -100,11 +100,12 @@ struct alignas(16) DevProxy {  // 128 B, read as 16-byte words
     float r2, h2_min, q2_max;  // r^2, (r cos_min)^2, squared outer radius of the shell
     float t_far;               // a first estimate of a crossing below this is behind the
                                // start (before its Newton step)
-    float gx, gy, gz, g2;      // sphere bounding the mesh: centre - c, squared radius
+    float gx, gy, gz, g2;      // sphere bounding the mesh: centre, squared radius
+    float g_r;                 // its radius
     int32_t surf;              // BVH reference of its surface when it has exactly one,
                                // else 0x7FFFFFFF
     float r;                   // radius, 0 for a plane
-    int32_t pad[2];
+    int32_t pad;
 };
 
 // Triangles (leaf positions) that a ray through the cell can meet: up to two

@@ -1309,7 +1309,9 @@ __device__ __noinline__ void nearest_bvh_far(const SceneView &sc, const DevNode 
 // instructions per RICH1 photon. Measured with the hits and fates the same:
 // trace of RICH1, 10^4 tracks, 1058 -> 725 us, of RICH2, 1.2 x 10^5 tracks,
 // 9.15 -> 6.01 ms, 10^6 caller photons on RICH1 463 -> 296 us a call.
-// Up to two crossings with cells are kept, nearest first (a third leaves the ray
+// A proxy whose mesh the ray passes by is left by one test of the sphere that
+// bounds it (RICH1, 10^4 tracks, 518 -> 485 us; RICH2 3.99 -> 3.78 ms). Up to two
+// crossings with cells are kept, nearest first (a third leaves the ray
 // to the BVH unless a nearer hit settles it), and their triangles are tested
 // after the last proxy, so that lanes whose mirrors differ test theirs together.
 template <bool EXT>
@@ -1331,28 +1333,27 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
         c0 = l0 ? c : c0;
         t0 = l0 ? t : t0;
     };
-    unsigned unsure = 0, entering = 0;
-    int i = 0;
+    unsigned entering = 0;
+    bool all = true;
 #pragma unroll 1
-    for (; i < sc.n_proxy_planes; ++i) {
+    for (int i = 0; i < S.n_proxies; ++i) {
         const DevProxy &P = S.proxies()[i];
+        if (proxy_misses(P, o.x, o.y, o.z, d.x, d.y, d.z, b.t) |
+            (P.surf == skip_ref & skip_ref != kNoSurf))
+            continue;
         float t;
         bool sure;
-        const int c = proxy_plane(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure);
-        const bool own = P.surf == skip_ref && skip_ref != kNoSurf;
-        unsure |= (unsigned)(!sure & !own) << i;
-        keep(t, own ? -1 : c);
-    }
-#pragma unroll 1
-    for (; i < S.n_proxies; ++i) {
-        const DevProxy &P = S.proxies()[i];
-        float t, sb, h2;
-        bool sure, ent;
-        const int c = proxy_sphere(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure, ent, sb, h2);
-        const bool own = P.surf == skip_ref && skip_ref != kNoSurf;
-        unsure |= (unsigned)(!sure & !own) << i;
-        entering |= (unsigned)(ent & !own) << i;
-        keep(t, own ? -1 : c);
+        int c;
+        if (i < sc.n_proxy_planes) {
+            c = proxy_plane(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure);
+        } else {
+            float sb, h2;
+            bool ent;
+            c = proxy_sphere(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure, ent, sb, h2);
+            entering |= (unsigned)ent << i;
+        }
+        all = all & sure;
+        keep(t, c);
     }
     while (entering) {                   // mostly the sphere just left
         const DevProxy &P = S.proxies()[__ffs(entering) - 1];
@@ -1365,12 +1366,6 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
         const int c = proxy_sphere_side(P, wx, wy, wz, d.x, d.y, d.z, sb, h2, -1.0f, t_min, b.t, t,
                                         true);
         keep(t, c);
-    }
-    bool all = true;
-    while (unsure) {
-        const DevProxy &P = S.proxies()[__ffs(unsure) - 1];
-        unsure &= unsure - 1u;
-        all = proxy_misses(P, o.x, o.y, o.z, d.x, d.y, d.z) && all;
     }
     if (c0 >= 0) {
         const Ray r = make_ray(o, d);

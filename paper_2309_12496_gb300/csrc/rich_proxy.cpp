@@ -203,15 +203,15 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     // sphere bounding the mesh, about the box's centre
     V3 g{};
     for (int k = 0; k < 3; ++k)
-        g[k] = 0.5 * (lo[0] + hi[0]) * e1[k] + 0.5 * (lo[1] + hi[1]) * e2[k] +
+        g[k] = f.c[k] + 0.5 * (lo[0] + hi[0]) * e1[k] + 0.5 * (lo[1] + hi[1]) * e2[k] +
                0.5 * (lo[2] + hi[2]) * axis[k];
     g = round32(g);
     double rho = 0.0;
     for (int i : f.tris)
-        for (int v = 0; v < 3; ++v) rho = std::max(rho, len(sub(sub(vert(T[i], v), f.c), g)));
+        for (int v = 0; v < 3; ++v) rho = std::max(rho, len(sub(vert(T[i], v), g)));
     // distances from c up to which the bounds are to hold (origins anywhere in
     // the scene's box), and the margins
-    const double W = o_max(extent) + len(f.c);
+    const double W = o_max(extent) + len(f.c), W_g = o_max(extent) + len(g);
     const double E = 32.0 * kUnit * W;
     const double margin = (f.shell + E) / kProxyCosMin + E;
     const double tri_size = std::sqrt(area / (double)f.tris.size());
@@ -248,7 +248,10 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     // 1e-6 t^2 / h, t <= 2 W and h >= r cos_min
     P.t_far = (float)(-(double)P.dt - (sphere ? 4.0e-6 * W * W / (f.r * kProxyCosMin) : 0.0));
     P.gx = (float)g[0]; P.gy = (float)g[1]; P.gz = (float)g[2];
-    P.g2 = (float)((rho + E + 4.0e-6 * W) * (rho + E + 4.0e-6 * W));
+    const double g_r = rho + E + P.dt + 4.0e-6 * W_g;
+    P.g_r = (float)(g_r * (1.0 + 1.0e-6));
+    // (a direction that is unit to 1e-6 changes (w . d)^2 by 2e-6 W^2 at most)
+    P.g2 = (float)((g_r * g_r + (16.0 * kUnit + 2.0e-6) * W_g * W_g) * (1.0 + 1.0e-6));
     P.surf = T[f.tris[0]].pad;
     for (int i : f.tris)
         if (T[i].pad != P.surf) P.surf = kNoSurf32;

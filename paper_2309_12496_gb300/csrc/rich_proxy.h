@@ -29,8 +29,7 @@ namespace rich {
 
 // The crossings of one ray with one proxy. cell >= 0: the cell to look up at
 // distance t; -1: the ray cannot meet the mesh there. sure: the margins hold
-// for this ray; if not, proxy_misses says whether the ray passes the mesh by
-// (else the BVH has to take it). t_max: the nearest hit known so far;
+// for this ray; if not, the BVH has to take it. t_max: the nearest hit known so far;
 // (dx, dy, dz) a unit vector to 1e-6, |o| at most the scene's o_max.
 //
 // The bounds: with u = 2^-24 and W >= |o - c|, the FP32 crossing point differs
@@ -39,9 +38,9 @@ namespace rich {
 // |p| = r, of |p|^2 - r^2), by 8 u W / c along the ray for an angle of
 // incidence with cosine c >= kProxyCosMin, and a facet's point lies within
 // `shell` of the surface; the cells' margin holds (shell + E) / kProxyCosMin + E
-// with E = 32 u W. The functions select instead of branching: a warp's rays
-// mostly take the same surfaces, and control flow was a fifth of the trace's
-// instructions.
+// with E = 32 u W. A crossing is found by selects instead of branches: a
+// warp's rays mostly take the same surfaces, and control flow was a fifth of the
+// trace's instructions.
 constexpr float kProxyCosMin = 0.25f;
 
 #ifdef __CUDA_ARCH__
@@ -51,6 +50,17 @@ RICH_HD float proxy_rsqrt(float a) { return rsqrtf(a); }
 RICH_HD float proxy_div(float a, float b) { return a / b; }
 RICH_HD float proxy_rsqrt(float a) { return 1.0f / sqrtf(a); }
 #endif
+
+// Whether the ray passes by the sphere that bounds the proxy's mesh, or meets it
+// beyond t_max or behind the start only. (|w|^2 - (w . d)^2 is off by at most
+// 16 u W^2, which g2 holds.)
+RICH_HD bool proxy_misses(const DevProxy &P, float ox, float oy, float oz, float dx, float dy,
+                          float dz, float t_max) {
+    const float wx = ox - P.gx, wy = oy - P.gy, wz = oz - P.gz;
+    const float w2 = fmaf(wx, wx, fmaf(wy, wy, wz * wz));
+    const float tb = -fmaf(wx, dx, fmaf(wy, dy, wz * dz));
+    return (fmaf(-tb, tb, w2) > P.g2) | ((tb < 0.0f) & (w2 > P.g2)) | (tb - P.g_r > t_max);
+}
 
 // The cell of the point p (relative to c) at distance t, or -1.
 RICH_HD int proxy_cell(const DevProxy &P, float px, float py, float pz, float t, float t_min,
@@ -106,15 +116,6 @@ RICH_HD int proxy_sphere(const DevProxy &P, float ox, float oy, float oz, float 
     const float far = -b - P.t_far;
     entering = meets & (far >= 0.0f) & (far * far >= h2);
     return proxy_sphere_side(P, wx, wy, wz, dx, dy, dz, b, h2, 1.0f, t_min, t_max, t, meets);
-}
-
-// Whether the ray passes by the sphere that bounds the proxy's mesh.
-RICH_HD bool proxy_misses(const DevProxy &P, float ox, float oy, float oz, float dx, float dy,
-                          float dz) {
-    const float gx = ox - P.cx - P.gx, gy = oy - P.cy - P.gy, gz = oz - P.cz - P.gz;
-    const float gb = fmaf(gx, dx, fmaf(gy, dy, gz * dz));
-    const float mx = fmaf(-gb, dx, gx), my = fmaf(-gb, dy, gy), mz = fmaf(-gb, dz, gz);
-    return fmaf(mx, mx, fmaf(my, my, mz * mz)) > P.g2;
 }
 
 // Host builder. On return `proxies` is empty when some triangle fits no

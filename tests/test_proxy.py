@@ -51,6 +51,7 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
             int cell[2] = {-1, -1};
             float t, b2, h2;
             bool sure, entering = false;
+            if (proxy_misses(P, O[0], O[1], O[2], D[0], D[1], D[2], t_max)) continue;
             if ((int)k < R.n_planes) {
                 cell[0] = proxy_plane(P, O[0], O[1], O[2], D[0], D[1], D[2], 1e-3f, t_max, t, sure);
             } else {
@@ -60,7 +61,7 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
                     cell[1] = proxy_sphere_side(P, O[0] - P.cx, O[1] - P.cy, O[2] - P.cz, D[0], D[1],
                                                 D[2], b2, h2, -1.0f, 1e-3f, t_max, t, true);
             }
-            if (!sure && !proxy_misses(P, O[0], O[1], O[2], D[0], D[1], D[2])) out[i] |= 2;
+            if (!sure) out[i] |= 2;
             for (int c : cell) {
                 if (c < 0) continue;
                 const DevProxyCell &L = R.cells[(size_t)c];
