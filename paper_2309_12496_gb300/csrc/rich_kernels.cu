@@ -963,12 +963,19 @@ __device__ __forceinline__ void nearest_rects(const SmemScene &S, f3 o, f3 d,
 #pragma unroll 1
     for (int k = 0; k < S.n_rects; ++k) {
         const DevRect &R = S.rects()[k];
-        if (R.prim == skip) continue;
         const f3 n = mk3(R.nx, R.ny, R.nz);
         const float den = dot3(d, n);
-        if (den == 0.0f) continue;
         const f3 oo = mk3(R.ox, R.oy, R.oz) - o;
-        const float t = __fdiv_rn(dot3(oo, n), den);
+        const float num = dot3(oo, n);
+        // one branch ahead of the division: the surface just left, a
+        // rectangle behind the start, and one beyond the nearest hit by more
+        // than the rounding of the quotient (the floor keeps the product's
+        // rounding out of the subnormal range): 6 rectangles of a scintillator
+        // box 808 -> 792 us, RICH1 analytic, 10^4 tracks, 593 -> 587 us
+        if ((R.prim == skip) | (num * den < 0.0f) |
+            (fabsf(num) > fmaxf(b.t * fabsf(den) * 1.000001f, 1.0e-30f)))
+            continue;
+        const float t = __fdiv_rn(num, den);
         if (!(t > t_min) || !(t < b.t)) continue;
         const f3 q = fma3(d, t, mk3(-oo.x, -oo.y, -oo.z));
         const float u = dot3(q, mk3(R.ux, R.uy, R.uz));
