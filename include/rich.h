@@ -296,8 +296,11 @@ typedef struct rich_trace_opts {
     int32_t blocks_per_sm;  /* resident blocks per SM of the persistent grid
                                (0 or above the occupancy limit -> the limit) */
     int32_t refill_min;     /* refill a warp when at least this many lanes are
-                               idle (1..32): the compaction interval          */
-    int32_t chunk;          /* photons a warp takes from the queue at a time */
+                               idle (1..32): the compaction interval (default
+                               32, or 16 in scenes of rectangles alone)      */
+    int32_t chunk;          /* photons a warp takes from the queue at a time
+                               (default 32, or 32..128 by what is left in
+                               scenes of rectangles alone)                   */
     int32_t wide_regs;      /* <= 256 threads: 0 caps the trace kernel at 64
                                registers (four blocks per SM), 1 uncapped;
                                257..896 threads: 1 caps it at 72 registers

@@ -234,6 +234,8 @@ struct TraceParams {
     int32_t precision, max_bounces, max_steps;
     float t_min;
     int32_t refill_min, chunk;
+    int32_t chunk_max, chunk_shift;   // > chunk: photons left >> shift are taken at a
+                              // time, between the two
     rich_hit *hits;
     uint64_t hit_capacity;
     uint32_t *pixel_counts;

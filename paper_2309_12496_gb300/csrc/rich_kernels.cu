@@ -1941,10 +1941,18 @@ k_trace(TraceArgs A) {
             uint64_t pool_next = wpool[0], pool_end = wpool[1];
             int64_t pool_track = (int64_t)wpool[2];
             const uint64_t N = EXT ? A.ext.n : (uint64_t)(*em.total);
-            const uint64_t chunk = (uint64_t)P.chunk;
+            uint64_t chunk = (uint64_t)P.chunk;
             while (idle != 0u && more) {
                 if (pool_next >= pool_end) {
                     unsigned long long base = 0;
+                    // guided: more at a time while much is left (the last chunks
+                    // stay small, so that the warps end together)
+                    if (P.chunk_max > P.chunk && pool_end != 0) {
+                        const uint64_t share = (N - pool_end) >> P.chunk_shift;
+                        chunk = share > (uint64_t)P.chunk_max ? (uint64_t)P.chunk_max
+                                                              : (share & ~31ull);
+                        chunk = chunk < (uint64_t)P.chunk ? (uint64_t)P.chunk : chunk;
+                    }
                     if (lane == 0) base = atomicAdd(&A.ctr->work, (unsigned long long)chunk);
                     base = __shfl_sync(kFull, base, 0);
                     if (base >= N) {
