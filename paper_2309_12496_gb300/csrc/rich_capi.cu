@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <array>
 #include <climits>
 #include <cmath>
 #include <cstdio>
@@ -179,6 +180,65 @@ bool finite3(const float *v) {
     return std::isfinite(v[0]) && std::isfinite(v[1]) && std::isfinite(v[2]);
 }
 
+// Sphere bounding tile s (FP64 centre g about the tile's own centre; returns the
+// radius). The tile's points are x e1 + y e2 + sqrt(r^2 - x^2 - y^2) axis over the
+// part of the cap's disc inside the edges, a convex set; the distance from a point
+// on the axis' side is a convex function of (x, y), largest at a corner of the
+// edges or on the circle, which is sampled (samples outside an edge by less than
+// their spacing count). Without an orthonormal frame the whole sphere bounds.
+double tile_bound(const rich_sphere &s, double g[3]) {
+    const double r = s.radius;
+    auto dot = [](const float *a, const float *b) {
+        return (double)a[0] * b[0] + (double)a[1] * b[1] + (double)a[2] * b[2];
+    };
+    for (int k = 0; k < 3; ++k) g[k] = 0.0;
+    bool frame = s.cos_min > 0.01f && s.cos_min < 1.0f;
+    const float *ax[3] = {s.e1, s.e2, s.axis};
+    for (int a = 0; a < 3; ++a)
+        for (int b = a; b < 3; ++b)
+            frame = frame && std::fabs(dot(ax[a], ax[b]) - (a == b ? 1.0 : 0.0)) < 1e-4;
+    if (!frame) return 1.001 * r;
+    const double cap = r * std::sqrt(1.0 - (double)s.cos_min * s.cos_min);
+    constexpr int kSamples = 64;
+    const double spacing = 2.0 * M_PI * cap / kSamples;
+    auto inside = [&](double x, double y, double slack) {
+        for (int e = 0; e < s.n_edges; ++e)
+            if (!(s.edges[e][0] * x + s.edges[e][1] * y <=
+                  s.edges[e][2] + slack * std::hypot(s.edges[e][0], s.edges[e][1])))
+                return false;
+        return true;
+    };
+    std::vector<std::pair<double, double>> at;
+    for (int a = 0; a < s.n_edges; ++a)
+        for (int b = a + 1; b < s.n_edges; ++b) {
+            const float *p = s.edges[a], *q = s.edges[b];
+            const double det = (double)p[0] * q[1] - (double)p[1] * q[0];
+            if (det == 0.0) continue;
+            const double x = ((double)p[2] * q[1] - (double)p[1] * q[2]) / det;
+            const double y = ((double)p[0] * q[2] - (double)p[2] * q[0]) / det;
+            if (std::hypot(x, y) <= cap && inside(x, y, 1e-5 * r)) at.push_back({x, y});
+        }
+    const size_t corners = at.size();
+    for (int k = 0; k < kSamples; ++k) {
+        const double x = cap * std::cos(2.0 * M_PI * k / kSamples);
+        const double y = cap * std::sin(2.0 * M_PI * k / kSamples);
+        if (inside(x, y, spacing)) at.push_back({x, y});
+    }
+    const double over = at.size() > corners ? spacing : 0.0;
+    if (at.empty()) return 1.001 * r;
+    auto point = [&](const std::pair<double, double> &q, int k) {
+        const double z = std::sqrt(std::max(0.0, r * r - q.first * q.first - q.second * q.second));
+        return q.first * s.e1[k] + q.second * s.e2[k] + z * s.axis[k];
+    };
+    for (const auto &q : at)
+        for (int k = 0; k < 3; ++k) g[k] += point(q, k) / (double)at.size();
+    double rad = 0.0;
+    for (const auto &q : at)
+        rad = std::max(rad, std::hypot(point(q, 0) - g[0], point(q, 1) - g[1], point(q, 2) - g[2]));
+    // the FP32 aperture tests and the frame's 1e-4
+    return rad + over + 1.0e-3 * r;
+}
+
 // Tiles sharing one sphere (identical FP32 centre and radius) form a group:
 // the sphere quadratic is solved once per group.
 bool group_tiles(const rich_sphere *sp, int n, int n_materials,
@@ -244,6 +304,22 @@ bool group_tiles(const rich_sphere *sp, int n, int n_materials,
             tiles.push_back(T);
         }
         G.count = (int)tiles.size() - G.first;
+        // one sphere around the bounds of its tiles
+        std::vector<std::array<double, 4>> bounds;
+        double mid[3] = {0.0, 0.0, 0.0}, rad = 0.0;
+        for (int t = G.first; t < G.first + G.count; ++t) {
+            std::array<double, 4> q;
+            q[3] = tile_bound(sp[tiles[t].prim], q.data());
+            bounds.push_back(q);
+            for (int k = 0; k < 3; ++k) mid[k] += q[k] / G.count;
+        }
+        for (const auto &q : bounds)
+            rad = std::max(rad, q[3] + std::hypot(q[0] - mid[0], q[1] - mid[1], q[2] - mid[2]));
+        G.gx = (float)(G.fcx + mid[0]);
+        G.gy = (float)(G.fcy + mid[1]);
+        G.gz = (float)(G.fcz + mid[2]);
+        rad += 1.0e-6 * (std::fabs(G.gx) + std::fabs(G.gy) + std::fabs(G.gz));
+        G.g2 = (float)(rad * rad * (1.0 + 1.0e-6));
     }
     return true;
 }

@@ -37,11 +37,12 @@ struct DevMaterial {
     int32_t kind, table, plane, flags;
 };
 
-struct DevSphereGroup {      // 32 B
+struct alignas(16) DevSphereGroup { // 48 B
     float fcx, fcy, fcz;     // the FP32 input centre
     float radius, inv_radius;
     int32_t first, count;    // tiles [first, first + count)
     float pad;
+    float gx, gy, gz, g2;    // sphere that bounds its tiles: centre, squared radius
 };
 
 struct DevTile {             // 160 B
