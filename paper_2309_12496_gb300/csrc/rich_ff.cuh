@@ -207,4 +207,97 @@ __device__ __forceinline__ ff3 ff3_reflect(ff3 d, ff3 n) {
     return ff3_axpy(k, n, d);
 }
 
+// ------------------------------------------------- fused forms (replays)
+// The refinement and gradient replays are bound by the number of FP32
+// operations (and the size of their straight-line code). A chain of the
+// accurate double-word additions above normalises after every term; these
+// forms take the leading parts' products and sums error-free (Ogita, Rump
+// and Oishi, "Accurate sum and dot product", SIAM J. Sci. Comput. 26(6), 2005)
+// and collect everything below them in one FP32 tail: 32 operations for a
+// three-term dot product instead of 67, 15 for a + s b instead of 29, with
+// errors of a few 2^-48 of the terms' sum in both.
+
+// x + t for a tail t below x's last place, as a double-word
+__device__ __forceinline__ ff ff_tail(float x, float t) { return fast_two_sum(x, t); }
+
+// low parts of the product x y: x.hi y.lo + x.lo y.hi + the rounding of
+// x.hi y.hi
+__device__ __forceinline__ float ff_cross(ff x, ff y, float p_lo) {
+    return __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, p_lo));
+}
+
+// a x + b y
+__device__ __forceinline__ ff ff_dot2(ff a, ff x, ff b, ff y) {
+    const ff p = two_prod(a.hi, x.hi), q = two_prod(b.hi, y.hi);
+    const ff s = two_sum(p.hi, q.hi);
+    return ff_tail(s.hi, __fadd_rn(s.lo, __fadd_rn(ff_cross(a, x, p.lo), ff_cross(b, y, q.lo))));
+}
+// a . b
+__device__ __forceinline__ ff ff_dot3(const ff3 &a, const ff3 &b) {
+    const ff p = two_prod(a.x.hi, b.x.hi), q = two_prod(a.y.hi, b.y.hi), r = two_prod(a.z.hi, b.z.hi);
+    const ff s = two_sum(p.hi, q.hi), t = two_sum(s.hi, r.hi);
+    return ff_tail(t.hi, __fadd_rn(__fadd_rn(s.lo, t.lo),
+                                   __fadd_rn(__fadd_rn(ff_cross(a.x, b.x, p.lo),
+                                                       ff_cross(a.y, b.y, q.lo)),
+                                             ff_cross(a.z, b.z, r.lo))));
+}
+// a . (bx, by, bz)
+__device__ __forceinline__ ff ff_dot3(const ff3 &a, float bx, float by, float bz) {
+    const ff p = two_prod(a.x.hi, bx), q = two_prod(a.y.hi, by), r = two_prod(a.z.hi, bz);
+    const ff s = two_sum(p.hi, q.hi), t = two_sum(s.hi, r.hi);
+    return ff_tail(t.hi, __fadd_rn(__fadd_rn(s.lo, t.lo),
+                                   __fadd_rn(__fadd_rn(__fmaf_rn(a.x.lo, bx, p.lo),
+                                                       __fmaf_rn(a.y.lo, by, q.lo)),
+                                             __fmaf_rn(a.z.lo, bz, r.lo))));
+}
+// a + s b
+__device__ __forceinline__ ff ff_axpy(ff s, ff b, ff a) {
+    const ff p = two_prod(s.hi, b.hi), t = two_sum(a.hi, p.hi);
+    return ff_tail(t.hi, __fadd_rn(t.lo, __fadd_rn(a.lo, ff_cross(s, b, p.lo))));
+}
+__device__ __forceinline__ ff3 ff3_axpy_fused(ff s, const ff3 &b, const ff3 &a) {
+    return {ff_axpy(s, b.x, a.x), ff_axpy(s, b.y, a.y), ff_axpy(s, b.z, a.z)};
+}
+// a - (bx, by, bz)
+__device__ __forceinline__ ff3 ff3_subf(const ff3 &a, float bx, float by, float bz) {
+    return {ff_add(a.x, -bx), ff_add(a.y, -by), ff_add(a.z, -bz)};
+}
+// The Newton corrections with one more order: the approximate reciprocals'
+// error (2^-22) enters to third order instead of second.
+__device__ __forceinline__ ff ff_div_newton(ff x, ff y) {
+    float ry = rcp_approx(y.hi);
+    ry = __fmaf_rn(ry, __fmaf_rn(-y.hi, ry, 1.0f), ry);
+    const float th = __fmul_rn(x.hi, ry);
+    // x - th y: the leading difference is exact
+    const ff p = two_prod(th, y.hi);
+    const float d = __fadd_rn(__fsub_rn(x.hi, p.hi), __fsub_rn(x.lo, __fmaf_rn(th, y.lo, p.lo)));
+    return fast_two_sum(th, __fmul_rn(d, ry));
+}
+__device__ __forceinline__ ff ff_sqrt_newton(ff x) {
+    if (!(x.hi > 0.0f)) return {0.0f, 0.0f};
+    float r = rsqrt_approx(x.hi);
+    r = __fmaf_rn(__fmul_rn(0.5f, r), __fmaf_rn(-__fmul_rn(x.hi, r), r, 1.0f), r);
+    const float s = __fmul_rn(x.hi, r);
+    const ff s2 = two_prod(s, s);
+    const float e = __fadd_rn(__fsub_rn(__fsub_rn(x.hi, s2.hi), s2.lo), x.lo);
+    return fast_two_sum(s, __fmul_rn(e, __fmul_rn(0.5f, r)));
+}
+__device__ __forceinline__ ff ff_rsqrt_newton(ff x) {
+    const float r = rsqrt_approx(x.hi);
+    const ff r2 = two_prod(r, r);
+    // 1 - x r^2: the leading product lies within 2^-21 of 1, so the
+    // difference is exact
+    const ff m = two_prod(x.hi, r2.hi);
+    const float e = __fsub_rn(__fsub_rn(1.0f, m.hi), __fmaf_rn(x.lo, r2.hi, __fmaf_rn(x.hi, r2.lo, m.lo)));
+    return fast_two_sum(r, __fmul_rn(__fmul_rn(r, e), __fmaf_rn(0.375f, e, 0.5f)));
+}
+__device__ __forceinline__ ff3 ff3_unit(const ff3 &a) {
+    return ff3_scale(a, ff_rsqrt_newton(ff_dot3(a, a)));
+}
+// reflection about the unit normal n: d - 2 (d.n) n
+__device__ __forceinline__ ff3 ff3_mirror(const ff3 &d, const ff3 &n) {
+    const ff k = ff_dot3(d, n);
+    return ff3_axpy_fused({-2.0f * k.hi, -2.0f * k.lo}, n, d);
+}
+
 }  // namespace rich

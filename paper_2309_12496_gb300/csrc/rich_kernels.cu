@@ -1414,6 +1414,13 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
 // extended past its edges, the final plane. All geometry is FP32 input, so
 // it enters the replay exactly. Runs in its own pass (k_refine), one thread
 // per stored hit, so the warps are converged.
+//
+// Meshes and planes, most of the replay's operations, use the fused forms; the
+// emission, sphere tiles and the final plane keep the chains of accurate
+// additions where their error is the larger part. Errors against 64 bits (rms
+// of the position, 1e-11 mm) before and after: RICH1 1.61 and 1.07, analytic 1.36
+// and 1.37, RICH2 2.91 and 2.48, windows 1.64 and 1.08, scintillator box 0.94 and
+// 0.88, water 1.05 and 1.01, point source 0.064 and 0.064.
 __device__ void replay_ff(const SceneView &sc, ff3 o, ff3 d, const RefineRec &rr, float lam,
                           ff &u, ff &v) {
     for (int k = 0; k < rr.n_path; ++k) {
@@ -1426,17 +1433,16 @@ __device__ void replay_ff(const SceneView &sc, ff3 o, ff3 d, const RefineRec &rr
             for (int q = 0; q < sc.n_tiles; ++q)
                 if (sc.tiles[q].prim == prim) ti = q;
             const DevSphereGroup &G = sc.groups[sc.tiles[ti].group];
-            const ff3 C = ff3v(G.fcx, G.fcy, G.fcz);
-            const ff3 w = ff3_sub(o, C);
+            const ff3 w = ff3_subf(o, G.fcx, G.fcy, G.fcz);
             const ff bq = ff3_dot(w, d);
             const ff c = ff_sub(ff3_dot(w, w), two_prod(G.radius, G.radius));
             const ff disc = ff_sub(ff_mul(bq, bq), c);
-            const ff sq = ff_sqrt(disc);
+            const ff sq = ff_sqrt_newton(disc);
             // concave (front) side: the exit root -b + sqrt(disc), taken in
             // the form free of cancellation
             const ff t = bq.hi <= 0.0f ? ff_sub(sq, bq) : ff_div(c, ff_sub(ff_neg(bq), sq));
             o = ff3_axpy(t, d, o);
-            const ff3 pc = ff3_sub(o, C);
+            const ff3 pc = ff3_subf(o, G.fcx, G.fcy, G.fcz);
             n = ff3_scale(pc, ff_neg(ff_rsqrt(ff3_dot(pc, pc))));
             ng = n;
             mat = sc.tiles[ti].material;
@@ -1445,7 +1451,8 @@ __device__ void replay_ff(const SceneView &sc, ff3 o, ff3 d, const RefineRec &rr
             n = ff3v(R.nx, R.ny, R.nz);
             ng = n;
             mat = R.material;
-            const ff t = ff_div(ff3_dot(ff3_sub(ff3v(R.ox, R.oy, R.oz), o), n), ff3_dot(d, n));
+            const ff t = ff_neg(ff_div_newton(ff_dot3(ff3_subf(o, R.ox, R.oy, R.oz), R.nx, R.ny, R.nz),
+                                              ff_dot3(d, R.nx, R.ny, R.nz)));
             o = ff3_axpy(t, d, o);
         } else {
             const int k_tri = prim - sc.tri_prim_base;   // leaf-order index
@@ -1454,10 +1461,10 @@ __device__ void replay_ff(const SceneView &sc, ff3 o, ff3 d, const RefineRec &rr
             // dot products), formed on the host in FP64
             const float4 *Q = reinterpret_cast<const float4 *>(sc.tri_ref + k_tri);
             const float4 q0 = __ldg(Q), q1 = __ldg(Q + 1);
-            const ff3 v0 = ff3v(T.v0x, T.v0y, T.v0z);
             ng = {ff{q0.x, q0.y}, ff{q0.z, q0.w}, ff{q1.x, q1.y}};
-            const ff t = ff_div(ff3_dot(ff3_sub(v0, o), ng), ff3_dot(d, ng));
-            o = ff3_axpy(t, d, o);
+            const ff3 w = ff3_subf(o, T.v0x, T.v0y, T.v0z);
+            const ff t = ff_neg(ff_div_newton(ff_dot3(w, ng), ff_dot3(d, ng)));
+            o = ff3_axpy_fused(t, d, o);
             mat = T.material;
             const DevMaterial &M = sc.materials[T.material];
             if ((M.flags & RICH_MAT_SMOOTH) && sc.tri_normals) {
@@ -1465,18 +1472,16 @@ __device__ void replay_ff(const SceneView &sc, ff3 o, ff3 d, const RefineRec &rr
                 const float4 q2 = __ldg(Q + 2), q3 = __ldg(Q + 3);
                 const ff3 e1 = ff3_diff(T.v1x, T.v1y, T.v1z, T.v0x, T.v0y, T.v0z);
                 const ff3 e2 = ff3_diff(T.v2x, T.v2y, T.v2z, T.v0x, T.v0y, T.v0z);
-                const ff3 q = ff3_sub(o, v0);
+                const ff3 q = ff3_subf(o, T.v0x, T.v0y, T.v0z);
                 const ff d00 = {q1.z, q1.w}, d01 = {q2.x, q2.y}, d11 = {q2.z, q2.w};
                 const ff inv_den = {q3.x, q3.y};
-                const ff d20 = ff3_dot(q, e1), d21 = ff3_dot(q, e2);
-                const ff b1 = ff_mul(ff_sub(ff_mul(d11, d20), ff_mul(d01, d21)), inv_den);
-                const ff b2 = ff_mul(ff_sub(ff_mul(d00, d21), ff_mul(d01, d20)), inv_den);
-                const ff b0 = ff_sub(ff_sub(ffv(1.0f), b1), b2);
+                const ff d20 = ff_dot3(q, e1), d21 = ff_dot3(q, e2);
+                const ff b1 = ff_mul(ff_dot2(d11, d20, ff_neg(d01), d21), inv_den);
+                const ff b2 = ff_mul(ff_dot2(d00, d21, ff_neg(d01), d20), inv_den);
+                const ff3 bc = {ff_sub(ff_sub(ffv(1.0f), b1), b2), b1, b2};
                 const float *N = sc.tri_normals + 9 * (int64_t)k_tri;
-                const ff3 m = ff3_add(ff3_add(ff3_scale(ff3v(N[0], N[1], N[2]), b0),
-                                              ff3_scale(ff3v(N[3], N[4], N[5]), b1)),
-                                      ff3_scale(ff3v(N[6], N[7], N[8]), b2));
-                n = ff3_normalized(m);
+                n = ff3_unit({ff_dot3(bc, N[0], N[3], N[6]), ff_dot3(bc, N[1], N[4], N[7]),
+                              ff_dot3(bc, N[2], N[5], N[8])});
             } else {
                 n = ng;
             }
@@ -1484,29 +1489,30 @@ __device__ void replay_ff(const SceneView &sc, ff3 o, ff3 d, const RefineRec &rr
         if (sc.materials[mat].kind == RICH_MAT_DIELECTRIC) {
             // refraction at a window face (as in the trace), double-word
             const float nw = table_eval(sc.tables[sc.materials[mat].table], lam);
-            const bool front = ff3_dot(d, ng).hi < 0.0f;
+            const bool front = ff_dot3(d, ng).hi < 0.0f;
             const ff3 N = front ? ng : ff3_scale(ng, -1.0f);
-            const ff eta = front ? ff_div(ffv(1.0f), ffv(nw)) : ffv(nw);
-            const ff c1 = ff_neg(ff3_dot(d, N));
+            const ff eta = front ? ff_div_newton(ffv(1.0f), ffv(nw)) : ffv(nw);
+            const ff c1 = ff_neg(ff_dot3(d, N));
             const ff kk = ff_sub(ffv(1.0f),
                                  ff_mul(ff_mul(eta, eta), ff_sub(ffv(1.0f), ff_mul(c1, c1))));
-            if (kk.hi < 0.0f)
-                d = ff3_reflect(d, N);
-            else
-                d = ff3_normalized(ff3_add(ff3_scale(d, eta),
-                                           ff3_scale(N, ff_sub(ff_mul(eta, c1), ff_sqrt(kk)))));
+            if (kk.hi < 0.0f) {
+                d = ff3_mirror(d, N);
+            } else {
+                const ff s = ff_sub(ff_mul(eta, c1), ff_sqrt_newton(kk));
+                d = ff3_unit({ff_dot2(d.x, eta, N.x, s), ff_dot2(d.y, eta, N.y, s),
+                              ff_dot2(d.z, eta, N.z, s)});
+            }
             continue;
         }
         // |d| = 1 is kept by the reflection about a unit normal
-        d = ff3_reflect(d, n);
+        d = prim < sc.n_tiles ? ff3_reflect(d, n) : ff3_mirror(d, n);
     }
     const DevRect &R = sc.rects[rr.det_rect];
-    const ff3 nrm = ff3v(R.nx, R.ny, R.nz);
-    const ff3 O = ff3v(R.ox, R.oy, R.oz);
-    const ff t = ff_div(ff3_dot(ff3_sub(O, o), nrm), ff3_dot(d, nrm));
-    const ff3 q = ff3_sub(ff3_axpy(t, d, o), O);
-    u = ff3_dot(q, R.ux, R.uy, R.uz);
-    v = ff3_dot(q, R.vx, R.vy, R.vz);
+    const ff3 w = ff3_subf(o, R.ox, R.oy, R.oz);
+    const ff t = ff_neg(ff_div_newton(ff_dot3(w, R.nx, R.ny, R.nz), ff_dot3(d, R.nx, R.ny, R.nz)));
+    const ff3 q = ff3_subf(ff3_axpy(t, d, o), R.ox, R.oy, R.oz);
+    u = ff_dot3(q, R.ux, R.uy, R.uz);
+    v = ff_dot3(q, R.vx, R.vy, R.vz);
 }
 
 // Orthonormal basis around a unit double-word vector (the branch-free form
@@ -1602,9 +1608,9 @@ __device__ void emit_ff(const TrackRec &tr, const TrackFrame &fr, float4 cs, uin
         ct = ff_from_double(cos_t);
         st = ff_from_double(nb1 > 0.0 ? sqrt(nb1 * (2.0 + nb1)) * cos_t : 0.0);
     }
-    d = ff3_normalized({ff_add(ff_mul(t.x, ct), ff_mul(r.x, st)),
-                        ff_add(ff_mul(t.y, ct), ff_mul(r.y, st)),
-                        ff_add(ff_mul(t.z, ct), ff_mul(r.z, st))});
+    const ff3 v = {ff_add(ff_mul(t.x, ct), ff_mul(r.x, st)), ff_add(ff_mul(t.y, ct), ff_mul(r.y, st)),
+                   ff_add(ff_mul(t.z, ct), ff_mul(r.z, st))};
+    d = ff3_normalized(v);
 }
 
 // Pixel of a double-word position: floor(u / pitch), clamped to the grid.
@@ -2325,9 +2331,12 @@ k_trace(TraceArgs A) {
 // Refinement pass: one thread per stored hit (converged warps). Hits are
 // taken in chunks of 32, chunk c by the warp with global index c over a
 // warp numbering that runs across the blocks first, so the chunks spread
-// evenly over the SMs whatever the hit count.
+// evenly over the SMs whatever the hit count. Bound by FP32 issue (two thirds of
+// its instructions are FP32 additions) and by instruction fetch at small counts.
+// With the fused forms and 32 warps per SM instead of 16, 5.0e5 RICH1 hits take 105
+// -> 80 us, 3.2e6 RICH2 hits 570 -> 436 us, 1.2e6 scintillator hits 268 -> 162 us.
 template <bool EXT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 4)
 k_refine(SceneView sc, EmitView em, ExtView ext, TraceParams P, Counters *ctr) {
     __shared__ double s_es_tab[kSmemKeys * 4];
     double *const s_es = es_table_on(sc, P) ? s_es_tab : nullptr;
@@ -2381,9 +2390,9 @@ cudaError_t launch_refine(const SceneView &sc, const EmitView *em, const ExtView
                           const TraceParams &p, Counters *counters, int n_sm,
                           cudaStream_t s) {
     if (p.hit_capacity == 0) return cudaSuccess;
-    // every block resident at once (two 256-thread blocks per SM)
+    // every block resident at once (four 256-thread blocks per SM)
     uint64_t blocks = (p.hit_capacity + 255) / 256;
-    const uint64_t cap = (uint64_t)n_sm * 2;
+    const uint64_t cap = (uint64_t)n_sm * 4;
     if (blocks > cap) blocks = cap;
     if (ext)
         return launch_pdl(k_refine<true>, (unsigned)blocks, 256, 0, s, sc,
