@@ -2335,12 +2335,28 @@ k_trace(TraceArgs A) {
 // its instructions are FP32 additions) and by instruction fetch at small counts.
 // With the fused forms and 32 warps per SM instead of 16, 5.0e5 RICH1 hits take 105
 // -> 80 us, 3.2e6 RICH2 hits 570 -> 436 us, 1.2e6 scintillator hits 268 -> 162 us.
+constexpr int kRefineThreads = 256;
+constexpr int kOwnKeys = 4;
 template <bool EXT>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(kRefineThreads, 4)
 k_refine(SceneView sc, EmitView em, ExtView ext, TraceParams P, Counters *ctr) {
     __shared__ double s_es_tab[kSmemKeys * 4];
     double *const s_es = es_table_on(sc, P) ? s_es_tab : nullptr;
     for (int i = threadIdx.x; i < kSmemKeys * 4; i += blockDim.x) s_es_tab[i] = 0.0;
+    // with few keys (one event) each thread sums its own hits, per key, and
+    // the warp's butterfly (15 double-word additions and shuffles per key) runs
+    // once at the end instead of once per chunk: 5.0e5 RICH1 hits 80 -> 63 us,
+    // 3.2e6 RICH2 hits 436 -> 337 us; more than four keys would take shared memory
+    // from the blocks beside this one
+    __shared__ ff s_own[kOwnKeys][3][kRefineThreads];
+    __shared__ uint32_t s_own_n[kOwnKeys][kRefineThreads];
+    const int n_keys = s_es ? (int)P.n_hist_events * sc.n_planes : 0;
+    const bool own = s_es && n_keys <= kOwnKeys;
+    if (own)
+        for (int k = 0; k < n_keys; ++k) {
+            for (int q = 0; q < 3; ++q) s_own[k][q][threadIdx.x] = ffv(0.0f);
+            s_own_n[k][threadIdx.x] = 0u;
+        }
     __syncthreads();
     grid_dep_wait();                     // the trace has ended
     const uint64_t n_hits = ctr->hits < P.hit_capacity ? ctr->hits : P.hit_capacity;
@@ -2380,7 +2396,33 @@ k_refine(SceneView sc, EmitView em, ExtView ext, TraceParams P, Counters *ctr) {
             lam = h.lambda;
             bin_hit(sc, P, event, plane, ix, iy);
         }
-        add_event_sums(sc, P, on, event, plane, uf, vf, lam, s_es);
+        if (!own) {
+            add_event_sums(sc, P, on, event, plane, uf, vf, lam, s_es);
+        } else if (on && event < P.n_hist_events) {
+            const int k = (int)event * sc.n_planes + plane;
+            ff(*a)[kRefineThreads] = s_own[k];
+            a[0][threadIdx.x] = ff_add(a[0][threadIdx.x], uf);
+            a[1][threadIdx.x] = ff_add(a[1][threadIdx.x], vf);
+            a[2][threadIdx.x] = ff_add(a[2][threadIdx.x], lam);
+            s_own_n[k][threadIdx.x] += 1u;
+        }
+    }
+    if (own) {
+        for (int k = 0; k < n_keys; ++k) {
+            const uint32_t n = __reduce_add_sync(kFull, s_own_n[k][threadIdx.x]);
+            if (n == 0) continue;        // uniform in the warp
+            ff a[3];
+#pragma unroll
+            for (int q = 0; q < 3; ++q) a[q] = s_own[k][q][threadIdx.x];
+#pragma unroll 1
+            for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+                for (int q = 0; q < 3; ++q) a[q] = ff_add(a[q], shfl_xor_ff(a[q], o));
+            if (lane == 0) {
+                atomicAdd(s_es + 4 * k, (double)n);
+                for (int q = 0; q < 3; ++q) atomicAdd(s_es + 4 * k + 1 + q, ff_to_double(a[q]));
+            }
+        }
     }
     __syncthreads();
     if (s_es) es_table_flush(sc, P, s_es);
@@ -2391,13 +2433,13 @@ cudaError_t launch_refine(const SceneView &sc, const EmitView *em, const ExtView
                           cudaStream_t s) {
     if (p.hit_capacity == 0) return cudaSuccess;
     // every block resident at once (four 256-thread blocks per SM)
-    uint64_t blocks = (p.hit_capacity + 255) / 256;
+    uint64_t blocks = (p.hit_capacity + kRefineThreads - 1) / kRefineThreads;
     const uint64_t cap = (uint64_t)n_sm * 4;
     if (blocks > cap) blocks = cap;
     if (ext)
-        return launch_pdl(k_refine<true>, (unsigned)blocks, 256, 0, s, sc,
+        return launch_pdl(k_refine<true>, (unsigned)blocks, kRefineThreads, 0, s, sc,
                           em ? *em : EmitView{}, *ext, p, counters);
-    return launch_pdl(k_refine<false>, (unsigned)blocks, 256, 0, s, sc, *em, ExtView{}, p,
+    return launch_pdl(k_refine<false>, (unsigned)blocks, kRefineThreads, 0, s, sc, *em, ExtView{}, p,
                       counters);
 }
 
