@@ -839,6 +839,8 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
             return fail(ctx, RICH_ERR_OOM, std::string("rich_init_geometry: proxies: ") + e.what());
         }
     }
+    for (size_t i = 0; i < tris.size() && !proxy.proxies.empty(); ++i)
+        tris[i].material |= (int32_t)(proxy.tri_code[i] << kTriProxyShift);
     std::vector<DevTable> tables(g->n_tables);
     for (int i = 0; i < g->n_tables; ++i) std::memcpy(&tables[i], &g->tables[i], sizeof(DevTable));
     std::vector<DevMaterial> mats(g->n_materials);
@@ -846,16 +848,18 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
 
     // ---- one device allocation
     auto r256 = [](size_t b) { return (b + 255) & ~size_t(255); };
+    size_t proxy_cell_bytes = 0;
+    for (const auto &grid : proxy.cells) proxy_cell_bytes += sizeof(DevProxyCell) * grid.size();
     size_t sizes[] = {sizeof(DevSphereGroup) * groups.size(), sizeof(DevTile) * tiles.size(),
                       sizeof(DevRect) * rects.size(), sizeof(DevTable) * tables.size(), sizeof(DevMaterial) * mats.size(),
                       sizeof(DevNode) * bvh.nodes.size(), sizeof(DevTri) * tris.size(),
                       sizeof(float) * normals.size(), sizeof(DevTriRef) * tri_ref.size(),
                       sizeof(DevProxy) * proxy.proxies.size(),
-                      sizeof(DevProxyCell) * proxy.cells.size(),
+                      proxy_cell_bytes,
                       sizeof(int32_t) * proxy.lists.size()};
     const void *srcs[] = {groups.data(), tiles.data(), rects.data(), tables.data(), mats.data(), bvh.nodes.data(), tris.data(),
                           normals.data(), tri_ref.data(), proxy.proxies.data(),
-                          proxy.cells.data(), proxy.lists.data()};
+                          nullptr, proxy.lists.data()};
     constexpr int kArrays = (int)(sizeof sizes / sizeof sizes[0]);
     size_t total = 0, offs[kArrays];
     for (int i = 0; i < kArrays; ++i) {
@@ -871,7 +875,16 @@ RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc 
     RICH_CUDA(cudaMalloc(&buf, std::max<size_t>(total, 256)));
     ctx->d_geom = buf;
     for (int i = 0; i < kArrays; ++i)
-        if (sizes[i]) RICH_CUDA(cudaMemcpy((char *)buf + offs[i], srcs[i], sizes[i], cudaMemcpyHostToDevice));
+        if (sizes[i] && srcs[i])
+            RICH_CUDA(cudaMemcpy((char *)buf + offs[i], srcs[i], sizes[i], cudaMemcpyHostToDevice));
+    {
+        char *grid_at = (char *)buf + offs[10];        // the proxies' grids one after another
+        for (const auto &grid : proxy.cells) {
+            const size_t bytes = sizeof(DevProxyCell) * grid.size();
+            RICH_CUDA(cudaMemcpy(grid_at, grid.data(), bytes, cudaMemcpyHostToDevice));
+            grid_at += bytes;
+        }
+    }
     SceneView sc{};
     auto at = [&](int i) { return sizes[i] ? (const void *)((char *)buf + offs[i]) : nullptr; };
     sc.groups = (const DevSphereGroup *)at(0);

@@ -63,11 +63,19 @@ struct DevRect {             // 80 B
     int32_t gx, gy, plane, prim;
 };
 
+// Proxy code of a triangle: the index of its surface proxy + 1 (0: none), and
+// whether the proxy holds its surface alone, or several of which no grid cell
+// lists two.
+constexpr int kTriProxyShift = 8;
+constexpr int kTriMaterialMask = 0xFF;
+constexpr uint32_t kProxyIndex = 0xF, kProxySingle = 0x10, kProxyApart = 0x20;
+
 struct alignas(16) DevTri {  // 48 B: v0 | v1 | v2 | prim, material, surface
     float v0x, v0y, v0z, v1x;
     float v1y, v1z, v2x, v2y;
     float v2z;
-    int32_t prim, material;
+    int32_t prim;
+    int32_t material;         // | proxy code << kTriProxyShift
     int32_t pad;              // BVH reference (node index or leaf code) of the
                               // subtree holding exactly this triangle's
                               // surface, or 0x7FFFFFFF when it has none
@@ -103,9 +111,8 @@ struct alignas(16) DevProxy {  // 128 B, read as 16-byte words
                                // start (before its Newton step)
     float gx, gy, gz, g2;      // sphere bounding the mesh: centre, squared radius
     float g_r;                 // its radius
-    int32_t surf;              // BVH reference of its surface when it has exactly one,
-                               // else 0x7FFFFFFF
     float r;                   // radius, 0 for a plane
+    int32_t code;              // kProxySingle or kProxyApart, or 0
     int32_t pad;
 };
 

@@ -701,7 +701,8 @@ struct Photon {
     uint32_t wr0, wr1, wr2, wr3;
     int skip, n_refl, steps;
     int n_turn;            // direction changes: reflections and refractions
-    int skip_ref;          // BVH subtree of the surface just left, or kNoSurf
+    int skip_ref;          // BVH subtree of the surface just left, or kNoSkip
+    uint32_t skip_px;      // proxy code (DevTri) of the triangle just left, or 0
 };
 
 // philox10 out of line, for the draw blocks that few photons need. A fifth of
@@ -1082,15 +1083,21 @@ __device__ __forceinline__ bool watertight(const Ray &r, const DevTri &T,
     return true;
 }
 
-__device__ __forceinline__ DevTri load_tri(const DevTri *p) {
+// A triangle record with its material and proxy code unpacked.
+struct Tri : DevTri {
+    uint32_t px;
+};
+
+__device__ __forceinline__ Tri load_tri(const DevTri *p) {
     const float4 *q = reinterpret_cast<const float4 *>(p);
     float4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
-    DevTri t;
+    Tri t;
     t.v0x = a.x; t.v0y = a.y; t.v0z = a.z; t.v1x = a.w;
     t.v1y = b.x; t.v1z = b.y; t.v2x = b.z; t.v2y = b.w;
     t.v2z = c.x;
     t.prim = __float_as_int(c.y);
-    t.material = __float_as_int(c.z);
+    t.material = __float_as_int(c.z) & kTriMaterialMask;
+    t.px = (uint32_t)__float_as_int(c.z) >> kTriProxyShift;
     t.pad = __float_as_int(c.w);
     return t;
 }
@@ -1151,7 +1158,7 @@ __device__ __forceinline__ void leaf_tris(const SceneView &sc, const Ray &r,
                                           Best &b, WorkTally *w) {
     const int first = code >> 3, count = (code & 7) + 1;
     for (int k = first; k < first + count; ++k) {
-        const DevTri T = load_tri(sc.tris + k);
+        const Tri T = load_tri(sc.tris + k);
         if (T.prim == skip) continue;
         if constexpr (COUNT) w->tris += 1;
         test_tri(sc, r, T, k, t_min, b);
@@ -1229,7 +1236,8 @@ __device__ __forceinline__ void cas_key(float &ka, int &ca, float &kb, int &cb) 
     ca = c;
 }
 
-constexpr int kNoSurf = 0x7FFFFFFF;   // no surface subtree to skip
+constexpr int kNoSurf = 0x7FFFFFFF;   // DevTri::pad of a triangle without a surface
+constexpr int kNoSkip = 0x7FFFFFFE;   // no surface subtree to skip (equal to no reference)
 
 // Nearest triangle along the ray: four-wide BVH in the "while-while" order
 // of Aila and Laine (HPG 2009): descend inner nodes (nearest child first, the
@@ -1334,7 +1342,8 @@ __device__ __noinline__ void nearest_bvh_far(const SceneView &sc, const DevNode 
 // after the last proxy, so that lanes whose mirrors differ test theirs together.
 template <bool EXT>
 __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemScene &S, f3 o, f3 d,
-                                                int skip, int skip_ref, float t_min, Best &b) {
+                                                int skip, int skip_ref, uint32_t skip_px,
+                                                float t_min, Best &b) {
     // origins outside the scene's box, and callers' directions that are not
     // unit vectors, are outside the proxies' bounds
     if (!(dot3(o, o) <= sc.proxy_o2_max)) return false;
@@ -1353,12 +1362,17 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
     };
     unsigned entering = 0;
     bool all = true;
+    // the proxy of the surface just left: passed over when that is its only
+    // surface; when its surfaces lie apart, its entry crossing (the start)
+    // lists none but the one left (RICH1, 10^4 tracks, 482 -> 457 us; RICH2 3.76
+    // -> 3.54 ms)
+    const int left = (int)(skip_px & kProxyIndex) - 1;
+    const int own = skip_px & kProxySingle ? left : -1;
+    const unsigned no_entry = skip_px & kProxyApart ? 1u << left : 0u;
 #pragma unroll 1
     for (int i = 0; i < S.n_proxies; ++i) {
         const DevProxy &P = S.proxies()[i];
-        if (proxy_misses(P, o.x, o.y, o.z, d.x, d.y, d.z, b.t) |
-            (P.surf == skip_ref & skip_ref != kNoSurf))
-            continue;
+        if (proxy_misses(P, o.x, o.y, o.z, d.x, d.y, d.z, b.t) | (i == own)) continue;
         float t;
         bool sure;
         int c;
@@ -1373,7 +1387,8 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
         all = all & sure;
         keep(t, c);
     }
-    while (entering) {                   // mostly the sphere just left
+    entering &= ~no_entry;
+    while (entering) {
         const DevProxy &P = S.proxies()[__ffs(entering) - 1];
         entering &= entering - 1u;
         const float wx = o.x - P.cx, wy = o.y - P.cy, wz = o.z - P.cz;
@@ -1395,8 +1410,8 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
 #pragma unroll 1
             for (int q = 0; q < n; ++q) {
                 const int tri = list ? __ldg(sc.proxy_lists + c.x + q) : (q ? c.y : c.x);
-                const DevTri T = load_tri(sc.tris + tri);
-                if (T.prim == skip || (T.pad == skip_ref && skip_ref != kNoSurf)) continue;
+                const Tri T = load_tri(sc.tris + tri);
+                if (T.prim == skip || T.pad == skip_ref) continue;
                 test_tri(sc, r, T, tri, t_min, b);
             }
             if (c1 < 0 || t1 > b.t + sc.proxy_dt) break;
@@ -1456,7 +1471,7 @@ __device__ void replay_ff(const SceneView &sc, ff3 o, ff3 d, const RefineRec &rr
             o = ff3_axpy(t, d, o);
         } else {
             const int k_tri = prim - sc.tri_prim_base;   // leaf-order index
-            const DevTri T = load_tri(sc.tris + k_tri);
+            const Tri T = load_tri(sc.tris + k_tri);
             // the triangle's refinement constants (unit normal, barycentric
             // dot products), formed on the host in FP64
             const float4 *Q = reinterpret_cast<const float4 *>(sc.tri_ref + k_tri);
@@ -1741,7 +1756,7 @@ __device__ __forceinline__ uint32_t refl_word(const Photon &ph, int k,
 // memory (a generic 64-bit pointer would hold two registers).
 enum : int {
     kCLam = 0, kCWqe, kCWr0, kCWr1, kCWr2, kCWr3, kCEvent, kCId, kCJ, kCGlo, kCGhi, kCTrack,
-    kCCount,            // n_refl | n_turn << 8 | steps << 16
+    kCCount,            // n_refl | n_turn << 8 | steps << 16 | skip_px << 24
     kColdWords
 };
 static_assert(kColdWords % 2 == 1, "an odd stride keeps the lanes in distinct banks");
@@ -1937,7 +1952,9 @@ k_trace(TraceArgs A) {
 #define PH_TRACK (kColdOn ? (uint32_t)cold.at(kCTrack) : ph.track)
 #define PH_NREFL (kColdOn ? (int)(cold.at(kCCount) & 0xFFu) : ph.n_refl)
 #define PH_NTURN (kColdOn ? (int)((cold.at(kCCount) >> 8) & 0xFFu) : ph.n_turn)
-#define PH_STEPS (kColdOn ? (int)(cold.at(kCCount) >> 16) : ph.steps)
+#define PH_STEPS (kColdOn ? (int)((cold.at(kCCount) >> 16) & 0xFFu) : ph.steps)
+#define PH_SKIP_PX (kColdOn ? (uint32_t)(cold.at(kCCount) >> 24) : ph.skip_px)
+#define PH_SET_SKIP_PX(px) do { if (kColdOn) cold.at(kCCount) = (cold.at(kCCount) & 0xFFFFFFu) | ((px) << 24); else ph.skip_px = (px); } while (0)
 #define PH_REFL_WORD(k) (kColdOn ? cold_refl_word(cold, (k), em) : refl_word(ph, (k), em))
 #define PH_ADD_REFL() do { if (kColdOn) cold.at(kCCount) = cold.at(kCCount) + 1u; else ph.n_refl += 1; } while (0)
 #define PH_ADD_TURN() do { if (kColdOn) cold.at(kCCount) = cold.at(kCCount) + 0x100u; else ph.n_turn += 1; } while (0)
@@ -2004,7 +2021,8 @@ k_trace(TraceArgs A) {
                     const uint64_t g = pool_next + (uint64_t)rank;
                     ph.g = g;
                     ph.skip = -1;
-                    ph.skip_ref = kNoSurf;
+                    ph.skip_ref = kNoSkip;
+                    ph.skip_px = 0u;
                     ph.n_refl = 0;
                     ph.n_turn = 0;
                     ph.steps = 0;
@@ -2109,7 +2127,8 @@ k_trace(TraceArgs A) {
                               ph.skip, P.t_min, b);
             nearest_rects(S, ph.o, ph.d, ph.skip, P.t_min, b);
             if constexpr (PROXY) {
-                if (!nearest_proxies<EXT>(sc, S, ph.o, ph.d, ph.skip, ph.skip_ref, P.t_min, b))
+                if (!nearest_proxies<EXT>(sc, S, ph.o, ph.d, ph.skip, ph.skip_ref, PH_SKIP_PX,
+                                          P.t_min, b))
                     nearest_bvh_far(sc, snodes, n_snodes, ph.o, ph.d, ph.skip, ph.skip_ref,
                                     P.t_min, b, A.ctr);
             } else if (has_tri)
@@ -2122,7 +2141,8 @@ k_trace(TraceArgs A) {
                 int mat_id;
                 bool front;
                 f3 n_sh, n_geo;
-                int hit_ref = kNoSurf;    // surface subtree of a hit triangle
+                int hit_ref = kNoSkip;    // surface subtree of a hit triangle
+                uint32_t hit_px = 0;      // and its proxy code
                 if (b.kind == 0) {
                     const DevTile &T = S.tiles()[b.idx];
                     const DevSphereGroup &G = S.groups()[T.group];
@@ -2137,14 +2157,15 @@ k_trace(TraceArgs A) {
                     front = dot3(ph.d, n_sh) < 0.0f;
                     mat_id = R.material;
                 } else {
-                    const DevTri T = load_tri(sc.tris + b.idx);
+                    const Tri T = load_tri(sc.tris + b.idx);
                     const f3 e1 = mk3(T.v1x - T.v0x, T.v1y - T.v0y, T.v1z - T.v0z);
                     const f3 e2 = mk3(T.v2x - T.v0x, T.v2y - T.v0y, T.v2z - T.v0z);
                     const f3 ng = cross3(e1, e2);
                     front = dot3(ph.d, ng) < 0.0f;
                     n_geo = normalize3(ng);
                     mat_id = T.material;
-                    hit_ref = T.pad;
+                    hit_ref = T.pad == kNoSurf ? kNoSkip : T.pad;
+                    hit_px = T.px;
                     const DevMaterial &M0 = S.materials()[mat_id];
                     if ((M0.flags & RICH_MAT_SMOOTH) && sc.tri_normals) {
                         const float *N3 = sc.tri_normals + 9 * (int64_t)b.idx;
@@ -2182,6 +2203,7 @@ k_trace(TraceArgs A) {
                             ph.o = p;
                             ph.skip = b.prim;
                             ph.skip_ref = hit_ref;
+                            if constexpr (PROXY) PH_SET_SKIP_PX(hit_px);
                         }
                     }
                 } else if (M.kind == RICH_MAT_DIELECTRIC) {
@@ -2204,12 +2226,14 @@ k_trace(TraceArgs A) {
                         ph.o = p;
                         ph.skip = b.prim;
                         ph.skip_ref = hit_ref;
+                        if constexpr (PROXY) PH_SET_SKIP_PX(hit_px);
                     }
                 } else {  // detector
                     if (!front) {
                         ph.o = p;
                         ph.skip = b.prim;
                         ph.skip_ref = hit_ref;
+                        if constexpr (PROXY) PH_SET_SKIP_PX(hit_px);
                     } else {
                         const bool pass =
                             P.n_prefilter || u24f(PH_WQE) < table_eval(S.tables()[M.table], PH_LAM);
@@ -2649,7 +2673,7 @@ __device__ void replay_dual(const SceneView &sc, const GradView &gv, const EmitV
             n = dm3_c(nn);
         } else {
             const int k_tri = prim - sc.tri_prim_base;
-            const DevTri T = load_tri(sc.tris + k_tri);
+            const Tri T = load_tri(sc.tris + k_tri);
             const float4 *Q = reinterpret_cast<const float4 *>(sc.tri_ref + k_tri);
             const float4 q0 = __ldg(Q), q1 = __ldg(Q + 1);
             const ff3 v0 = ff3v(T.v0x, T.v0y, T.v0z);

@@ -24,13 +24,12 @@ using V3 = std::array<double, 3>;
 constexpr double kUnit = 1.0 / 16777216.0;   // 2^-24
 constexpr int32_t kNoSurf32 = 0x7FFFFFFF;
 // Cells of a quarter of the root mean triangle area: most list one triangle.
-// Trace of RICH1, 10^4 tracks, with cells of 1, 0.5, 0.35, 0.25 of it: 835,
-// 774, 749, 725 us; of RICH2, 1.2 x 10^5 tracks: 7.33, 6.55, 6.28, 6.01 ms
-// (0.15 gains 5 % on RICH1 for twice the building time). A cell is at least
-// four margins wide, and there are at most kMaxCellsPerTri cells a triangle
-// (meshes whose bounding rectangle is mostly empty get larger cells).
+// A cell is at least four margins wide; there are at most kMaxCellsPerTri cells a
+// triangle (meshes whose bounding rectangle is mostly empty get larger cells) and
+// kMaxCells in all (96 MB, which the L2 holds).
 constexpr double kCellScale = 0.25;
 constexpr double kMaxCellsPerTri = 64.0;
+constexpr double kMaxCells = 1.2e7;
 
 V3 vert(const DevTri &t, int k) {
     return k == 0 ? V3{t.v0x, t.v0y, t.v0z}
@@ -217,7 +216,8 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     const double tri_size = std::sqrt(area / (double)f.tris.size());
     double size = std::max(kCellScale * tri_size, 4.0 * margin);
     const double wx = hi[0] - lo[0] + 4.0 * margin, wy = hi[1] - lo[1] + 4.0 * margin;
-    const double most = kMaxCellsPerTri * (double)f.tris.size() + 4096.0;
+    const double share = (double)f.tris.size() / (double)T.size();
+    const double most = std::min(kMaxCellsPerTri * (double)f.tris.size(), kMaxCells * share) + 4096.0;
     if (wx * wy > most * size * size) size = std::sqrt(wx * wy / most);
     // long thin meshes: no more than `most` cells along either side
     size = std::max(size, std::max(wx, wy) / most);
@@ -252,13 +252,19 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     P.g_r = (float)(g_r * (1.0 + 1.0e-6));
     // (a direction that is unit to 1e-6 changes (w . d)^2 by 2e-6 W^2 at most)
     P.g2 = (float)((g_r * g_r + (16.0 * kUnit + 2.0e-6) * W_g * W_g) * (1.0 + 1.0e-6));
-    P.surf = T[f.tris[0]].pad;
-    for (int i : f.tris)
-        if (T[i].pad != P.surf) P.surf = kNoSurf32;
-    // the triangles whose projection comes within the margin of each cell:
-    // separating-axis test of the triangle's edges and the widened cell
-    std::vector<std::pair<int32_t, int32_t>> found;       // (cell, triangle)
-    std::vector<int32_t> start((size_t)nx * ny + 1, 0);
+    // the triangles whose projection comes within the margin of each cell (the
+    // triangle's edges and the widened cell, by separating axes), row by row
+    // the first two triangles of a cell go into it, further ones aside
+    std::vector<DevProxyCell> &cells = out.cells[0];
+    cells.assign((size_t)nx * ny, DevProxyCell{-1, -1});
+    std::vector<std::pair<int32_t, int32_t>> more;        // (cell, triangle)
+    // one surface, or several apart: a photon that leaves a facet starts within
+    // the margin of it, so the cell of its start lists that facet's surface
+    bool single = true, apart = true;
+    for (int i : f.tris) {
+        single = single && T[i].pad == T[f.tris[0]].pad;
+        apart = apart && T[i].pad != kNoSurf32;
+    }
     for (int i : f.tris) {
         double q[3][2], blo[2] = {HUGE_VAL, HUGE_VAL}, bhi[2] = {-HUGE_VAL, -HUGE_VAL};
         for (int v = 0; v < 3; ++v) {
@@ -273,43 +279,63 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
         const double turn = (q[1][0] - q[0][0]) * (q[2][1] - q[0][1]) -
                             (q[1][1] - q[0][1]) * (q[2][0] - q[0][0]);
         const double sg = turn < 0.0 ? -1.0 : 1.0;
-        const int ix0 = std::max(0, (int)std::floor(blo[0]));
         const int iy0 = std::max(0, (int)std::floor(blo[1]));
-        const int ix1 = std::min(nx - 1, (int)std::floor(bhi[0]));
         const int iy1 = std::min(ny - 1, (int)std::floor(bhi[1]));
         const double half = 0.5 + m;
-        for (int iy = iy0; iy <= iy1; ++iy)
-            for (int ix = ix0; ix <= ix1; ++ix) {
-                const double mx = ix + 0.5, my = iy + 0.5;
-                bool apart = false;
-                for (int v = 0; v < 3 && !apart; ++v) {
-                    const double *a = q[v], *b = q[(v + 1) % 3];
-                    const double ex = sg * (b[1] - a[1]), ey = -sg * (b[0] - a[0]);   // outward
-                    apart = ex * (mx - a[0]) + ey * (my - a[1]) >
-                            (std::fabs(ex) + std::fabs(ey)) * half;
-                }
-                if (apart) continue;
-                found.push_back({iy * nx + ix, i});
-                start[(size_t)iy * nx + ix + 1] += 1;
-            }
-    }
-    for (size_t c = 1; c < start.size(); ++c) start[c] += start[c - 1];
-    std::vector<int32_t> sorted(found.size()), at(start.begin(), start.end() - 1);
-    for (const auto &[c, i] : found) sorted[(size_t)at[(size_t)c]++] = i;
-    for (size_t k = 0; k + 1 < start.size(); ++k) {
-        const int32_t *l = sorted.data() + start[k];
-        const int32_t n = start[k + 1] - start[k];
-        DevProxyCell c{-1, -1};
-        if (n <= 2) {
-            if (n > 0) c.a = l[0];
-            if (n > 1) c.b = l[1];
-        } else {
-            c.a = (int32_t)out.lists.size();
-            c.b = (int32_t)(0x80000000u | (uint32_t)n);
-            out.lists.insert(out.lists.end(), l, l + n);
+        // outward normal of each edge and the bound of its half plane, widened
+        // by the cell
+        double ex[3], ey[3], rhs[3];
+        for (int v = 0; v < 3; ++v) {
+            const double *a = q[v], *b = q[(v + 1) % 3];
+            ex[v] = sg * (b[1] - a[1]);
+            ey[v] = -sg * (b[0] - a[0]);
+            rhs[v] = (std::fabs(ex[v]) + std::fabs(ey[v])) * half * (1.0 + 1.0e-9) + ex[v] * a[0] +
+                     ey[v] * a[1];
         }
-        out.cells.push_back(c);
+        for (int iy = iy0; iy <= iy1; ++iy) {
+            // the cells of a row that meet the triangle are consecutive
+            const double my = iy + 0.5;
+            double lo_x = blo[0] - 0.5, hi_x = bhi[0] + 0.5;       // of the cell's centre
+            for (int v = 0; v < 3; ++v) {
+                const double r = rhs[v] - ey[v] * my;
+                if (ex[v] > 0.0)
+                    hi_x = std::min(hi_x, r / ex[v]);
+                else if (ex[v] < 0.0)
+                    lo_x = std::max(lo_x, r / ex[v]);
+                else if (r < 0.0)
+                    hi_x = -1.0;
+            }
+            const int ix0 = std::max(0, (int)std::ceil(lo_x - 0.5 - 1.0e-6));
+            const int ix1 = std::min(nx - 1, (int)std::floor(hi_x - 0.5 + 1.0e-6));
+            DevProxyCell *row = cells.data() + (size_t)iy * nx;
+            for (int ix = ix0; ix <= ix1; ++ix) {
+                DevProxyCell &d = row[ix];
+                if (d.a < 0) {
+                    d.a = i;
+                    continue;
+                }
+                apart = apart && T[d.a].pad == T[i].pad;
+                if (d.b < 0)
+                    d.b = i;
+                else
+                    more.push_back({iy * nx + ix, i});
+            }
+        }
     }
+    std::sort(more.begin(), more.end());
+    for (size_t k = 0; k < more.size();) {
+        DevProxyCell &d = cells[(size_t)more[k].first];
+        const size_t first = out.lists.size();
+        out.lists.push_back(d.a);
+        out.lists.push_back(d.b);
+        out.list_cells.push_back(more[k].first);
+        const int32_t cell = more[k].first;
+        for (; k < more.size() && more[k].first == cell; ++k) out.lists.push_back(more[k].second);
+        d.a = (int32_t)first;
+        d.b = (int32_t)(0x80000000u | (uint32_t)(out.lists.size() - first));
+    }
+    if (T[f.tris[0]].pad != kNoSurf32)
+        P.code = single ? (int32_t)kProxySingle : (apart ? (int32_t)kProxyApart : 0);
     out.proxies.push_back(P);
     return true;
 }
@@ -365,21 +391,25 @@ void build_proxies(const std::vector<DevTri> &T, double extent, ProxyResult &out
     std::vector<ProxyResult> part(fits.size());
     run_parallel(fits.size(), [&](size_t k) {
         Fit &f = fits[k];
+        part[k].cells.resize(1);
         const bool ok = f.r > 0.0 ? fit_sphere(T, f.tris, f) : fit_plane(T, f.tris, f);
         if (!ok || !make_proxy(T, f, extent, part[k])) part[k] = ProxyResult();
     });
-    for (const ProxyResult &p : part) {
-        if (p.proxies.empty() || out.cells.size() + p.cells.size() > (size_t)2e8) {
+    out.tri_code.assign(T.size(), 0u);
+    size_t n_cells = 0;
+    for (ProxyResult &p : part) {
+        if (p.proxies.empty() || n_cells + p.cells[0].size() > (size_t)2e8) {
             out = ProxyResult();
             return;
         }
+        for (int i : fits[out.proxies.size()].tris)
+            out.tri_code[i] = (uint32_t)p.proxies[0].code | (uint32_t)(out.proxies.size() + 1);
         out.proxies.push_back(p.proxies[0]);
-        out.proxies.back().first_cell = (int32_t)out.cells.size();
-        for (DevProxyCell c : p.cells) {
-            if (c.b < -1) c.a += (int32_t)out.lists.size();
-            out.cells.push_back(c);
-        }
+        out.proxies.back().first_cell = (int32_t)n_cells;
+        for (int32_t cell : p.list_cells) p.cells[0][(size_t)cell].a += (int32_t)out.lists.size();
         out.lists.insert(out.lists.end(), p.lists.begin(), p.lists.end());
+        n_cells += p.cells[0].size();
+        out.cells.push_back(std::move(p.cells[0]));
         out.n_planes += p.proxies[0].r == 0.0f;
         out.dt_max = std::max(out.dt_max, p.proxies[0].dt);
     }

@@ -122,8 +122,10 @@ RICH_HD int proxy_sphere(const DevProxy &P, float ox, float oy, float oz, float 
 // proxy (the scene then uses the BVH alone).
 struct ProxyResult {
     std::vector<DevProxy> proxies;
-    std::vector<DevProxyCell> cells;
+    std::vector<std::vector<DevProxyCell>> cells;   // one grid per proxy, in order
     std::vector<int32_t> lists;       // triangle lists of the cells with more than two
+    std::vector<int32_t> list_cells;  // (while building) those cells
+    std::vector<uint32_t> tri_code;   // proxy code of every triangle
     int n_planes = 0;                 // planes first, then spheres
     float o2_max = 0.0f;              // |o|^2 up to which the bounds hold
     float dt_max = 0.0f;              // largest dt of any proxy

@@ -64,7 +64,7 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
             if (!sure) out[i] |= 2;
             for (int c : cell) {
                 if (c < 0) continue;
-                const DevProxyCell &L = R.cells[(size_t)c];
+                const DevProxyCell &L = R.cells[k][(size_t)(c - P.first_cell)];
                 const bool list = L.b < -1;
                 const int n = list ? (L.b & 0x7FFFFFFF) : (L.a >= 0) + (L.b >= 0);
                 tests += n;
