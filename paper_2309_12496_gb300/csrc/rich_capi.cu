@@ -120,6 +120,8 @@ struct rich_ctx {
     // gradient: nominal tiles (host), their frames (device), tilted copies
     std::vector<rich_sphere> nom_spheres;
     void *d_grad_tiles = nullptr;          // groups + tiles + tile duals at theta
+    void *h_grad_tiles = nullptr;          // pinned copy, and whether it may be in flight
+    bool grad_tiles_busy = false;
     double *d_acc = nullptr;               // 12 FP64 accumulators
     double *h_acc = nullptr;               // pinned
     // captured emit + trace (CUDA graph) and the stream it was captured on
@@ -625,6 +627,7 @@ RICH_API rich_status rich_destroy(rich_ctx *ctx) {
         cudaFree(ctx->d_geom);
         cudaFree(ctx->d_refine);
         cudaFree(ctx->d_grad_tiles);
+        cudaFreeHost(ctx->h_grad_tiles);
         for (RunSlot &S : ctx->run_slots) {
             cudaFreeHost(S.h_ctr);
             cudaFree(S.d_tracks);
@@ -1334,21 +1337,24 @@ RICH_API rich_status rich_trace_grad(rich_ctx *ctx, const rich_tracks *t,
         std::string gerr;
         if (!group_tiles(at.data(), ns, ctx->sc.n_materials, groups, tiles, gerr))
             return fail(ctx, RICH_ERR_ARG, "rich_trace_grad: " + gerr);
+        // one copy from pinned memory, not waited for: the call ends with a
+        // synchronisation (a call that failed before it leaves the flag set)
+        if (!ctx->h_grad_tiles) RICH_CUDA(cudaMallocHost(&ctx->h_grad_tiles, grad_tiles_bytes()));
+        if (ctx->grad_tiles_busy) RICH_CUDA(cudaDeviceSynchronize());
+        char *stage = static_cast<char *>(ctx->h_grad_tiles);
         char *base = static_cast<char *>(ctx->d_grad_tiles);
-        RICH_CUDA(cudaMemcpyAsync(base, groups.data(), sizeof(DevSphereGroup) * groups.size(),
-                                  cudaMemcpyHostToDevice, ctx->stream));
-        char *tb = base + sizeof(DevSphereGroup) * RICH_MAX_GROUPS;
-        RICH_CUDA(cudaMemcpyAsync(tb, tiles.data(), sizeof(DevTile) * tiles.size(),
-                                  cudaMemcpyHostToDevice, ctx->stream));
-        char *db = tb + sizeof(DevTile) * RICH_MAX_TILES;
-        RICH_CUDA(cudaMemcpyAsync(db, duals.data(), sizeof(DevTileDual) * ns,
-                                  cudaMemcpyHostToDevice, ctx->stream));
-        grad_duals = reinterpret_cast<const DevTileDual *>(db);
+        const size_t at_tiles = sizeof(DevSphereGroup) * groups.size();
+        const size_t at_duals = at_tiles + sizeof(DevTile) * tiles.size();
+        const size_t bytes = at_duals + sizeof(DevTileDual) * duals.size();
+        std::memcpy(stage, groups.data(), at_tiles);
+        std::memcpy(stage + at_tiles, tiles.data(), at_duals - at_tiles);
+        std::memcpy(stage + at_duals, duals.data(), bytes - at_duals);
+        ctx->grad_tiles_busy = true;
+        RICH_CUDA(cudaMemcpyAsync(base, stage, bytes, cudaMemcpyHostToDevice, ctx->stream));
+        grad_duals = reinterpret_cast<const DevTileDual *>(base + at_duals);
         sv.groups = reinterpret_cast<const DevSphereGroup *>(base);
-        sv.tiles = reinterpret_cast<const DevTile *>(tb);
+        sv.tiles = reinterpret_cast<const DevTile *>(base + at_tiles);
         sv.n_groups = (int)groups.size();
-        // host vectors must outlive the asynchronous copies
-        RICH_CUDA(cudaStreamSynchronize(ctx->stream));
     }
     {
         rich_status st = emit_core(ctx, t, prm->seed, th->n_minus_1, prm->lambda_min,
@@ -1430,6 +1436,7 @@ RICH_API rich_status rich_trace_grad(rich_ctx *ctx, const rich_tracks *t,
     RICH_CUDA(cudaMemcpyAsync(ctx->h_ctr, ctx->d_ctr, kCtrBytes, cudaMemcpyDeviceToHost,
                               ctx->stream));
     RICH_CUDA(cudaStreamSynchronize(ctx->stream));
+    ctx->grad_tiles_busy = false;
     ctx->traced = true;
     ctx->last_ext = false;
     ctx->last_capacity = hit_cap;

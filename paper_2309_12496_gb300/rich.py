@@ -8,6 +8,7 @@ and fails loudly when the library is missing (there is no CPU fallback).
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 import threading
 
@@ -767,16 +768,16 @@ def rich_version() -> str:
     return load().rich_version().decode()
 
 
-def ring_chi2(ctx: Context, theta, tracks: DeviceTracks, targets, outputs: TraceOutputs,
-              sigma=1.0, seed=0):
-    """Differentiable soft ring chi^2: a torch.autograd.Function over the
-    10 parameters (8 tile tilts, radius of curvature, n - 1); its backward
-    is the gradient from rich_trace_grad's adjoint pass."""
+@functools.lru_cache(maxsize=None)
+def _ring_chi2_function():
+    """The autograd function of ring_chi2 (made once: torch is imported on
+    first use, and making the class on every call took longer than the rest
+    of the call's host work)."""
     torch = _torch()
 
     class _RingChi2(torch.autograd.Function):
         @staticmethod
-        def forward(fctx, th):
+        def forward(fctx, th, ctx, tracks, targets, outputs, sigma, seed):
             loss, grad, used = ctx.trace_grad(tracks, th.detach().cpu().tolist(), targets,
                                               outputs, sigma=sigma, seed=seed)
             fctx.save_for_backward(torch.tensor(grad, dtype=th.dtype, device=th.device))
@@ -786,9 +787,17 @@ def ring_chi2(ctx: Context, theta, tracks: DeviceTracks, targets, outputs: Trace
         @staticmethod
         def backward(fctx, gout):
             (grad,) = fctx.saved_tensors
-            return gout * grad
+            return gout * grad, None, None, None, None, None, None
 
-    return _RingChi2.apply(theta)
+    return _RingChi2
+
+
+def ring_chi2(ctx: Context, theta, tracks: DeviceTracks, targets, outputs: TraceOutputs,
+              sigma=1.0, seed=0):
+    """Differentiable soft ring chi^2: a torch.autograd.Function over the
+    10 parameters (8 tile tilts, radius of curvature, n - 1); its backward
+    is the gradient from rich_trace_grad's adjoint pass."""
+    return _ring_chi2_function().apply(theta, ctx, tracks, targets, outputs, sigma, seed)
 
 
 def rich_trace_grad(ctx: Context, tracks, theta, targets, outputs, **kw):
