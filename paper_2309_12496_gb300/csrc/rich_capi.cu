@@ -67,7 +67,14 @@ struct rich_ctx {
     TrackFrame *d_frame = nullptr;
     uint32_t *d_counts = nullptr;
     uint64_t *d_offsets = nullptr;
+    // group sums of the photon counts in two slots: an emission sums into one
+    // and its yield kernel zeroes the other (whose reader has ended by then) for
+    // the next, so no reset sits before the kernel; used[k]: entries of slot k
+    // that may not be zero
     unsigned long long *d_bsum = nullptr;
+    int64_t bsum_stride = 0;
+    int bsum_slot = 0;
+    int64_t bsum_used[2] = {0, 0};
     bool has_emission = false;
     int64_t n_tracks = 0;
     // azimuth order of each track's photons (sized from the last photon
@@ -104,6 +111,8 @@ struct rich_ctx {
     // counting build of the trace (rich_trace_work): 6 device tallies
     unsigned long long *d_work = nullptr;
     int graph_slot = 0;
+    int graph_bsum_slot = 0;              // the captured emission's group sums
+    int64_t graph_bsum_used = 0;
     Counters *h_ctr = nullptr;            // pinned
     unsigned long long *h_total = nullptr; // pinned
     // last trace
@@ -466,7 +475,11 @@ rich_status emit_core(rich_ctx *ctx, const rich_tracks *t, uint64_t seed, float 
         RICH_CUDA(cudaMalloc(&ctx->d_frame, sizeof(TrackFrame) * cap));
         RICH_CUDA(cudaMalloc(&ctx->d_counts, sizeof(uint32_t) * cap));
         RICH_CUDA(cudaMalloc(&ctx->d_offsets, sizeof(uint64_t) * (cap + 1)));
-        RICH_CUDA(cudaMalloc(&ctx->d_bsum, sizeof(unsigned long long) * (blocks + 1)));
+        RICH_CUDA(cudaMalloc(&ctx->d_bsum, sizeof(unsigned long long) * 2 * (blocks + 1)));
+        RICH_CUDA(cudaMemsetAsync(ctx->d_bsum, 0, sizeof(unsigned long long) * 2 * (blocks + 1),
+                                  ctx->stream));
+        ctx->bsum_stride = blocks + 1;
+        ctx->bsum_used[0] = ctx->bsum_used[1] = 0;
         ctx->track_cap = cap;
     }
     ctx->key0 = (uint32_t)seed;
@@ -486,19 +499,33 @@ rich_status emit_core(rich_ctx *ctx, const rich_tracks *t, uint64_t seed, float 
         RICH_CUDA(cudaMemsetAsync(ctx->d_total, 0, sizeof(unsigned long long), ctx->stream));
         RICH_CUDA(cudaMemsetAsync(ctx->d_offsets, 0, sizeof(uint64_t), ctx->stream));
     } else {
+        // (a captured emission resets its own slot: its replays sum into it again)
+        const int64_t groups = (n + yield_block_threads() - 1) / yield_block_threads();
+        const int slot = ctx->bsum_slot ^ 1, other = ctx->bsum_slot;
+        const bool clear = ctx->capturing || ctx->bsum_used[slot] != 0;
+        if (clear && ctx->bsum_used[slot] > groups && !ctx->capturing)
+            RICH_CUDA(cudaMemsetAsync(ctx->d_bsum + slot * ctx->bsum_stride, 0,
+                                      sizeof(unsigned long long) * ctx->bsum_used[slot],
+                                      ctx->stream));
+        unsigned long long *const zero =
+            ctx->capturing ? nullptr : ctx->d_bsum + other * ctx->bsum_stride;
+        const int64_t n_zero = ctx->capturing ? 0 : ctx->bsum_used[other];
+        ctx->bsum_used[slot] = ctx->capturing ? std::max(ctx->bsum_used[slot], groups) : groups;
+        ctx->bsum_slot = slot;
         RICH_CUDA(launch_yield(tv, (double)n_minus_1, lambda_min, lambda_max, ctx->key0,
-                               ctx->key1, ctx->d_rec, ctx->d_cs, ctx->d_counts, ctx->d_bsum,
-                               ctx->stream,
+                               ctx->key1, ctx->d_rec, ctx->d_cs, ctx->d_counts,
+                               ctx->d_bsum + slot * ctx->bsum_stride, ctx->stream,
                                YieldModel{source == RICH_SOURCE_ISOTROPIC ? (double)yield_per_mm
                                                                           : -1.0,
                                           dispersion, disp_a, disp_lambda0},
-                               ctx->d_frame, ctx->d_perm_ok));
+                               ctx->d_frame, ctx->d_perm_ok, clear, zero, n_zero));
+        if (!ctx->capturing) ctx->bsum_used[other] = 0;
         // deferred: the ordering pass (order_photons, which the caller
         // runs next) does the scan
         ctx->scan_pending = defer_scan && n <= kOrderScanMaxTracks;
         if (!ctx->scan_pending)
-            RICH_CUDA(launch_offsets(ctx->d_counts, ctx->d_bsum, n, ctx->d_offsets,
-                                     ctx->d_total, ctx->stream));
+            RICH_CUDA(launch_offsets(ctx->d_counts, ctx->d_bsum + slot * ctx->bsum_stride, n,
+                                     ctx->d_offsets, ctx->d_total, ctx->stream));
     }
     ctx->n_tracks = n;
     ctx->source = source;
@@ -550,7 +577,8 @@ rich_status order_photons(rich_ctx *ctx) {
         RICH_CUDA(cudaMemsetAsync(ctx->d_perm_ok, 0, sizeof(uint32_t), ctx->stream));
         return RICH_OK;
     }
-    const OrderScan scan{ctx->d_counts, ctx->d_bsum, ctx->d_offsets, ctx->d_total};
+    const OrderScan scan{ctx->d_counts, ctx->d_bsum + ctx->bsum_slot * ctx->bsum_stride,
+                         ctx->d_offsets, ctx->d_total};
     RICH_CUDA(launch_order(em, ctx->d_perm, ctx->perm_cap, ctx->d_perm_ok, ctx->n_sm,
                            ctx->stream, ctx->scan_pending ? &scan : nullptr));
     ctx->scan_pending = false;
@@ -983,6 +1011,14 @@ RICH_API rich_status rich_emit(rich_ctx *ctx, const rich_tracks *t,
                                          /*defer_scan=*/!(n_photons || out));
         if (st != RICH_OK) return st;
     }
+    // the arrays are written before the host reads the total, so the GPU does not
+    // wait for it (arrays that are missing or too small are refused below,
+    // unwritten)
+    const bool arrays = out && out->x && out->y && out->z && out->dx && out->dy && out->dz &&
+                        out->lambda && out->event && out->track && out->photon;
+    if (arrays)
+        RICH_CUDA(launch_materialize(ctx->sc, emit_view(ctx), out->capacity, *out, ctx->n_sm,
+                                     ctx->stream));
     if (n_photons || out) {
         RICH_CUDA(cudaMemcpyAsync(ctx->h_total, ctx->d_total, sizeof(unsigned long long),
                                   cudaMemcpyDeviceToHost, ctx->stream));
@@ -1005,11 +1041,8 @@ RICH_API rich_status rich_emit(rich_ctx *ctx, const rich_tracks *t,
             return fail(ctx, RICH_ERR_OVERFLOW, "rich_emit: photon capacity " +
                                                     std::to_string(out->capacity) + " < " +
                                                     std::to_string(total));
-        if (total && (!out->x || !out->y || !out->z || !out->dx || !out->dy || !out->dz ||
-                      !out->lambda || !out->event || !out->track || !out->photon))
+        if (total && !arrays)
             return fail(ctx, RICH_ERR_ARG, "rich_emit: a photon output array is NULL");
-        const EmitView em = emit_view(ctx);
-        RICH_CUDA(launch_materialize(ctx->sc, em, total, *out, ctx->stream));
         out->n = total;
     }
     return RICH_OK;
@@ -1683,6 +1716,8 @@ RICH_API rich_status rich_graph_capture(rich_ctx *ctx, const rich_tracks *t,
     if (st == RICH_OK) st = rich_trace(ctx, nullptr, o, out);
     ctx->capturing = false;
     ctx->graph_slot = ctx->cur_slot;
+    ctx->graph_bsum_slot = ctx->bsum_slot;
+    ctx->graph_bsum_used = ctx->bsum_used[ctx->bsum_slot];
     cudaGraph_t g = nullptr;
     const cudaError_t e = cudaStreamEndCapture(ctx->stream, &g);
     ctx->stream = user;
@@ -1704,6 +1739,8 @@ RICH_API rich_status rich_graph_launch(rich_ctx *ctx) {
     RICH_CUDA(cudaGraphLaunch(ctx->graph_exec, ctx->stream));
     // the replay counted into the captured slot; the other one is not known
     // to be zero
+    ctx->bsum_used[ctx->graph_bsum_slot] =
+        std::max(ctx->bsum_used[ctx->graph_bsum_slot], ctx->graph_bsum_used);
     ctx->cur_slot = ctx->graph_slot;
     ctx->d_ctr = ctx->d_ctr_slot[ctx->graph_slot];
     ctx->slot_zeroed[ctx->graph_slot] = false;

@@ -292,12 +292,16 @@ struct LaunchShape {
 // model.iso_yield >= 0: isotropic source with that mean per mm (the
 // Cherenkov angle is not computed); < 0: Cherenkov source, constant index
 // n_minus_1 or the dispersive radiator of model.
+// clear: the group sums (block_sums) are zeroed first, else they are zero;
+// zero, n_zero: words that the kernel zeroes for a later call.
 cudaError_t launch_yield(const TracksView &t, double n_minus_1,
                          double lam_min, double lam_max, uint32_t key0,
                          uint32_t key1, TrackRec *rec, float4 *cs,
                          uint32_t *counts, unsigned long long *block_sums,
                          cudaStream_t s, const YieldModel &model,
-                         TrackFrame *frame = nullptr, uint32_t *perm_ok = nullptr);
+                         TrackFrame *frame = nullptr, uint32_t *perm_ok = nullptr,
+                         bool clear = true, unsigned long long *zero = nullptr,
+                         int64_t n_zero = 0);
 cudaError_t launch_offsets(const uint32_t *counts,
                            const unsigned long long *block_sums,
                            int64_t n_tracks, uint64_t *offsets,
@@ -320,8 +324,9 @@ struct OrderScan {
 };
 cudaError_t launch_order(const EmitView &em, uint2 *perm, uint64_t cap, uint32_t *perm_ok,
                          int n_sm, cudaStream_t s, const OrderScan *scan = nullptr);
+// Photons as arrays; nothing when the device's photon total exceeds capacity.
 cudaError_t launch_materialize(const SceneView &sc, const EmitView &em,
-                               uint64_t n, const rich_photons &out,
+                               uint64_t capacity, const rich_photons &out, int n_sm,
                                cudaStream_t s);
 // counters: the trace's slot (the kernel also stores the photon total right
 // after it); next: the slot it zeroes for the next trace, or null.
