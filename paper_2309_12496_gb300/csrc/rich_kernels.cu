@@ -703,10 +703,11 @@ struct Photon {
     uint64_t g;            // global photon index
     uint32_t w_qe;
     uint32_t wr0, wr1, wr2, wr3;
-    int skip, n_refl, steps;
-    int n_turn;            // direction changes: reflections and refractions
+    int skip;
+    uint32_t count;        // reflections | direction changes (reflections and refractions)
+                           // << 8 | steps << 16 | skip_px << 24, skip_px the proxy code
+                           // (DevTri) of the triangle just left, or 0
     int skip_ref;          // BVH subtree of the surface just left, or kNoSkip
-    uint32_t skip_px;      // proxy code (DevTri) of the triangle just left, or 0
 };
 
 // philox10 out of line, for the draw blocks that few photons need. A fifth of
@@ -1805,7 +1806,7 @@ __device__ __forceinline__ uint32_t refl_word(const Photon &ph, int k,
 // memory (a generic 64-bit pointer would hold two registers).
 enum : int {
     kCLam = 0, kCWqe, kCWr0, kCWr1, kCWr2, kCWr3, kCEvent, kCId, kCJ, kCGlo, kCGhi, kCTrack,
-    kCCount,            // n_refl | n_turn << 8 | steps << 16 | skip_px << 24
+    kCCount,            // Photon::count
     kColdWords
 };
 static_assert(kColdWords % 2 == 1, "an odd stride keeps the lanes in distinct banks");
@@ -1988,15 +1989,13 @@ k_trace(TraceArgs A) {
 #define PH_J (kColdOn ? (uint32_t)cold.at(kCJ) : ph.j)
 #define PH_G (kColdOn ? (((uint64_t)cold.at(kCGhi) << 32) | cold.at(kCGlo)) : ph.g)
 #define PH_TRACK (kColdOn ? (uint32_t)cold.at(kCTrack) : ph.track)
-#define PH_NREFL (kColdOn ? (int)(cold.at(kCCount) & 0xFFu) : ph.n_refl)
-#define PH_NTURN (kColdOn ? (int)((cold.at(kCCount) >> 8) & 0xFFu) : ph.n_turn)
-#define PH_STEPS (kColdOn ? (int)((cold.at(kCCount) >> 16) & 0xFFu) : ph.steps)
-#define PH_SKIP_PX (kColdOn ? (uint32_t)(cold.at(kCCount) >> 24) : ph.skip_px)
-#define PH_SET_SKIP_PX(px) do { if (kColdOn) cold.at(kCCount) = (cold.at(kCCount) & 0xFFFFFFu) | ((px) << 24); else ph.skip_px = (px); } while (0)
+    // the photon's counts and proxy code, one word read when the nearest surface is
+    // known and written back at the step's end: n_refl | n_turn << 8 | steps << 16 | skip_px << 24
+#define PH_NREFL ((int)(cnt & 0xFFu))
+#define PH_NTURN ((int)((cnt >> 8) & 0xFFu))
+#define PH_STEPS ((int)((cnt >> 16) & 0xFFu))
+#define PH_COUNT (kColdOn ? (uint32_t)cold.at(kCCount) : ph.count)
 #define PH_REFL_WORD(k) (kColdOn ? cold_refl_word(cold, (k), em) : refl_word(ph, (k), em))
-#define PH_ADD_REFL() do { if (kColdOn) cold.at(kCCount) = cold.at(kCCount) + 1u; else ph.n_refl += 1; } while (0)
-#define PH_ADD_TURN() do { if (kColdOn) cold.at(kCCount) = cold.at(kCCount) + 0x100u; else ph.n_turn += 1; } while (0)
-#define PH_ADD_STEP() do { if (kColdOn) cold.at(kCCount) = cold.at(kCCount) + 0x10000u; else ph.steps += 1; } while (0)
     // the warp's photon pool (next, end, track of next; warp-uniform) lives
     // in shared memory between refills, so that it holds no registers
     // through the bounce loop
@@ -2060,10 +2059,7 @@ k_trace(TraceArgs A) {
                     ph.g = g;
                     ph.skip = -1;
                     ph.skip_ref = kNoSkip;
-                    ph.skip_px = 0u;
-                    ph.n_refl = 0;
-                    ph.n_turn = 0;
-                    ph.steps = 0;
+                    ph.count = 0u;
                     if (EXT) {
                         ph.track = (uint32_t)g;
                         ph.lam = A.ext.lambda[g];
@@ -2152,6 +2148,7 @@ k_trace(TraceArgs A) {
         int fate = 0;
         int det_rect = -1;
         float hit_u = 0.0f, hit_v = 0.0f;
+        uint32_t cnt = 0;
         if (alive) {
             Best b;
             b.t = 3.0e38f;
@@ -2165,13 +2162,14 @@ k_trace(TraceArgs A) {
                               ph.skip, P.t_min, b);
             nearest_rects(S, ph.o, ph.d, ph.skip, P.t_min, b);
             if constexpr (PROXY) {
-                if (!nearest_proxies<EXT>(sc, S, ph.o, ph.d, ph.skip, ph.skip_ref, PH_SKIP_PX,
+                if (!nearest_proxies<EXT>(sc, S, ph.o, ph.d, ph.skip, ph.skip_ref, PH_COUNT >> 24,
                                           P.t_min, b))
                     nearest_bvh_far(sc, snodes, n_snodes, ph.o, ph.d, ph.skip, ph.skip_ref,
                                     P.t_min, b, A.ctr);
             } else if (has_tri)
                 nearest_bvh<COUNT>(sc, snodes, n_snodes, ph.o, ph.d, ph.skip, ph.skip_ref,
                                    P.t_min, b, A.ctr, COUNT ? &tally : nullptr);
+            cnt = PH_COUNT;
             if (b.prim < 0) {
                 fate = RICH_FATE_ESCAPED;
             } else {
@@ -2236,12 +2234,12 @@ k_trace(TraceArgs A) {
                             ph.d = normalize3(reflect_f(ph.d, n_sh));
                             if constexpr (COUNT) tally.turns += 1;
                             if (REFINE) path[PH_NTURN] = b.kind == 2 ? sc.tri_prim_base + b.idx : b.prim;
-                            PH_ADD_REFL();
-                            PH_ADD_TURN();
+                            cnt += 1u;
+                            cnt += 0x100u;
                             ph.o = p;
                             ph.skip = b.prim;
                             ph.skip_ref = hit_ref;
-                            if constexpr (PROXY) PH_SET_SKIP_PX(hit_px);
+                            if constexpr (PROXY) cnt = (cnt & 0xFFFFFFu) | hit_px << 24;
                         }
                     }
                 } else if (M.kind == RICH_MAT_DIELECTRIC) {
@@ -2260,18 +2258,18 @@ k_trace(TraceArgs A) {
                                         : normalize3(fma3(N, eta * c1 - sqrtf(k), ph.d * eta));
                         if constexpr (COUNT) tally.turns += 1;
                         if (REFINE) path[PH_NTURN] = b.kind == 2 ? sc.tri_prim_base + b.idx : b.prim;
-                        PH_ADD_TURN();
+                        cnt += 0x100u;
                         ph.o = p;
                         ph.skip = b.prim;
                         ph.skip_ref = hit_ref;
-                        if constexpr (PROXY) PH_SET_SKIP_PX(hit_px);
+                        if constexpr (PROXY) cnt = (cnt & 0xFFFFFFu) | hit_px << 24;
                     }
                 } else {  // detector
                     if (!front) {
                         ph.o = p;
                         ph.skip = b.prim;
                         ph.skip_ref = hit_ref;
-                        if constexpr (PROXY) PH_SET_SKIP_PX(hit_px);
+                        if constexpr (PROXY) cnt = (cnt & 0xFFFFFFu) | hit_px << 24;
                     } else {
                         const bool pass =
                             P.n_prefilter || u24f(PH_WQE) < table_eval(S.tables()[M.table], PH_LAM);
@@ -2288,8 +2286,12 @@ k_trace(TraceArgs A) {
                     }
                 }
                 if (fate == 0) {
-                    PH_ADD_STEP();
+                    cnt += 0x10000u;
                     if (PH_STEPS >= P.max_steps) fate = RICH_FATE_MAX_STEPS;
+                    if (kColdOn)
+                        cold.at(kCCount) = cnt;
+                    else
+                        ph.count = cnt;
                 }
             }
         }
