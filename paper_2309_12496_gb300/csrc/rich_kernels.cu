@@ -559,6 +559,41 @@ constexpr int kOrderWarps = 4;
 // 8 warps per block were slower on 10^4 tracks)
 constexpr uint32_t kOrderBinCache = 8192;
 
+// The photon total; SCAN: also the exclusive prefix of the 256-track group sums,
+// in s_gpre (one entry per group), by the whole block.
+template <bool SCAN, int WARPS>
+__device__ __forceinline__ uint64_t order_prefix(const EmitView &em, const OrderScan &scan,
+                                                 unsigned long long *s_gpre) {
+    if (!SCAN) return *em.total;
+    __shared__ unsigned long long s_wsum[WARPS];
+    __shared__ unsigned long long s_total;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // a contiguous segment of groups per thread, then a block scan of
+    // the segment sums
+    const int ng = (int)((em.n_tracks + kYieldThreads - 1) / kYieldThreads);
+    const int per = (ng + (int)blockDim.x - 1) / (int)blockDim.x;
+    const int a = min((int)threadIdx.x * per, ng), b = min(a + per, ng);
+    unsigned long long seg = 0;
+    for (int g = a; g < b; ++g) seg += scan.group_sums[g];
+    unsigned long long inc = seg;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(kFull, inc, o);
+        if (lane >= o) inc += y;
+    }
+    if (lane == 31) s_wsum[w] = inc;
+    __syncthreads();
+    unsigned long long run = inc - seg;
+    for (int k = 0; k < w; ++k) run += s_wsum[k];
+    for (int g = a; g < b; ++g) {
+        s_gpre[g] = run;
+        run += scan.group_sums[g];
+    }
+    if (threadIdx.x == blockDim.x - 1) s_total = run;
+    __syncthreads();
+    return s_total;
+}
+
 // SCAN: the offsets are not computed yet; each block first forms the
 // exclusive prefix of the 256-track group sums in shared memory, and each
 // track's warp adds the counts before it in its group and writes its
@@ -566,45 +601,12 @@ constexpr uint32_t kOrderBinCache = 8192;
 template <bool SCAN>
 __global__ void __launch_bounds__(32 * kOrderWarps) k_order(EmitView em, uint2 *perm,
                                                             uint64_t cap, uint32_t *perm_ok,
-                                                            OrderScan scan, bool signal_early) {
+                                                            OrderScan scan) {
     grid_dep_wait();                     // the yield (and scan) pass has ended
-    // the trace's prologue may start, when every block orders one track;
-    // over many tracks per block the trace's blocks, resident early, slowed
-    // the ordering pass (RICH2, 4.9e5 tracks: 45 -> 50 ms per chunk)
-    if (signal_early) grid_dep_launch_dependents();
+    grid_dep_launch_dependents();        // the trace's prologue may start
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     extern __shared__ unsigned long long s_gpre[];      // SCAN: one entry per group
-    __shared__ unsigned long long s_wsum[kOrderWarps];
-    __shared__ unsigned long long s_total;
-    uint64_t total;
-    if (SCAN) {
-        // a contiguous segment of groups per thread, then a block scan of
-        // the segment sums
-        const int ng = (int)((em.n_tracks + kYieldThreads - 1) / kYieldThreads);
-        const int per = (ng + (int)blockDim.x - 1) / (int)blockDim.x;
-        const int a = min((int)threadIdx.x * per, ng), b = min(a + per, ng);
-        unsigned long long seg = 0;
-        for (int g = a; g < b; ++g) seg += scan.group_sums[g];
-        unsigned long long inc = seg;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(kFull, inc, o);
-            if (lane >= o) inc += y;
-        }
-        if (lane == 31) s_wsum[w] = inc;
-        __syncthreads();
-        unsigned long long run = inc - seg;
-        for (int k = 0; k < w; ++k) run += s_wsum[k];
-        for (int g = a; g < b; ++g) {
-            s_gpre[g] = run;
-            run += scan.group_sums[g];
-        }
-        if (threadIdx.x == blockDim.x - 1) s_total = run;
-        __syncthreads();
-        total = s_total;
-    } else {
-        total = *em.total;
-    }
+    const uint64_t total = order_prefix<SCAN, kOrderWarps>(em, scan, s_gpre);
     const bool fits = total <= cap;
     // perm_ok (zeroed by the yield pass): bit 0 the entries fit the buffer,
     // bit 1 a track above kOrderMaxPhotons kept index order (its entries are
@@ -617,81 +619,189 @@ __global__ void __launch_bounds__(32 * kOrderWarps) k_order(EmitView em, uint2 *
         }
     }
     if (!SCAN && !fits) return;
-    // one block per track (grid-stride): the block's warps share the bin
-    // histogram, so each lane draws and places only a few photons
+    // the block's warps share the track's bin histogram, so each lane draws and
+    // places only a few photons
     __shared__ uint32_t hist[kAzBins];
     __shared__ uint8_t bins[kOrderBinCache];
     __shared__ unsigned long long s_part[kOrderWarps];
     const int nthreads = (int)blockDim.x;
-    for (int64_t t = blockIdx.x; t < em.n_tracks; t += gridDim.x) {   // block-uniform
-        uint64_t off, n64;
-        if (SCAN) {
-            const int64_t g = t / kYieldThreads;
-            unsigned long long part = 0;
-            for (int64_t i = g * kYieldThreads + threadIdx.x; i < t; i += nthreads)
-                part += scan.counts[i];
+    const int64_t t = blockIdx.x;
+    uint64_t off, n64;
+    if (SCAN) {
+        const int64_t g = t / kYieldThreads;
+        unsigned long long part = 0;
+        for (int64_t i = g * kYieldThreads + threadIdx.x; i < t; i += nthreads)
+            part += scan.counts[i];
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
-            if (lane == 0) s_part[w] = part;
-            __syncthreads();
-            off = s_gpre[g];
-            for (int k = 0; k < kOrderWarps; ++k) off += s_part[k];
-            n64 = scan.counts[t];
-            if (threadIdx.x == 0) scan.offsets[t] = off;
-        } else {
-            off = em.offsets[t];
-            n64 = em.offsets[t + 1] - off;
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
+        if (lane == 0) s_part[w] = part;
+        __syncthreads();
+        off = s_gpre[g];
+        for (int k = 0; k < kOrderWarps; ++k) off += s_part[k];
+        n64 = scan.counts[t];
+        if (threadIdx.x == 0) scan.offsets[t] = off;
+    } else {
+        off = em.offsets[t];
+        n64 = em.offsets[t + 1] - off;
+    }
+    if (fits && n64 > kOrderMaxPhotons && threadIdx.x == 0) atomicOr(perm_ok, 2u);
+    if (fits && n64 != 0 && n64 <= kOrderMaxPhotons) {   // uniform in the block
+        const uint32_t n = (uint32_t)n64;
+        const uint32_t id = em.tracks[t].id, ev = em.tracks[t].event;
+        if (threadIdx.x < kAzBins) hist[threadIdx.x] = 0u;
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < n; j += (uint32_t)nthreads) {
+            const uint32_t bin = philox10(0u, j, id, ev, em.key0, em.key1).y >> 27;
+            if (j < kOrderBinCache) bins[j] = (uint8_t)bin;
+            atomicAdd(&hist[bin], 1u);
         }
-        if (fits && n64 > kOrderMaxPhotons && threadIdx.x == 0) atomicOr(perm_ok, 2u);
-        if (fits && n64 != 0 && n64 <= kOrderMaxPhotons) {   // uniform in the block
-            const uint32_t n = (uint32_t)n64;
-            const uint32_t id = em.tracks[t].id, ev = em.tracks[t].event;
-            if (threadIdx.x < kAzBins) hist[threadIdx.x] = 0u;
-            __syncthreads();
-            for (uint32_t j = threadIdx.x; j < n; j += (uint32_t)nthreads) {
-                const uint32_t bin = philox10(0u, j, id, ev, em.key0, em.key1).y >> 27;
-                if (j < kOrderBinCache) bins[j] = (uint8_t)bin;
-                atomicAdd(&hist[bin], 1u);
-            }
-            __syncthreads();
-            if (w == 0) {
-                const uint32_t c = hist[lane];
-                uint32_t inc = c;
+        __syncthreads();
+        if (w == 0) {
+            const uint32_t c = hist[lane];
+            uint32_t inc = c;
 #pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const uint32_t y = __shfl_up_sync(kFull, inc, o);
-                    if (lane >= o) inc += y;
-                }
-                hist[lane] = inc - c;                           // bin cursors
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += y;
             }
-            __syncthreads();
-            for (uint32_t j = threadIdx.x; j < n; j += (uint32_t)nthreads) {
-                const uint32_t bin = j < kOrderBinCache
-                                         ? (uint32_t)bins[j]
-                                         : philox10(0u, j, id, ev, em.key0, em.key1).y >> 27;
-                perm[off + atomicAdd(&hist[bin], 1u)] = make_uint2(j, (uint32_t)t);
-            }
+            hist[lane] = inc - c;                           // bin cursors
         }
-        __syncthreads();                 // the shared histogram and bins are reused
+        __syncthreads();
+        for (uint32_t j = threadIdx.x; j < n; j += (uint32_t)nthreads) {
+            const uint32_t bin = j < kOrderBinCache
+                                     ? (uint32_t)bins[j]
+                                     : philox10(0u, j, id, ev, em.key0, em.key1).y >> 27;
+            perm[off + atomicAdd(&hist[bin], 1u)] = make_uint2(j, (uint32_t)t);
+        }
     }
 }
 
+// The same with one warp per track and a run of consecutive tracks per warp, for
+// emissions of many tracks: no block barriers, the offsets carried from track to
+// track, and each photon's rank in its bin kept from the counting pass. A block
+// per track is the shorter chain for few tracks, but waits on its six barriers:
+// 2.5e7 photons of 1.2e5 RICH2 tracks 171 -> 103 us (29 us of them the 8 bytes
+// written per photon).
+constexpr int kOrderBlocksPerSm = 64;
+constexpr int kOrderRunWarps = 8;
+constexpr uint32_t kOrderRunCache = 2048;   // photons whose bin and rank are kept
+static_assert(kOrderRunCache <= (1u << 11), "a kept rank takes 11 bits of its word");
+template <bool SCAN>
+__global__ void __launch_bounds__(32 * kOrderRunWarps) k_order_run(EmitView em, uint2 *perm,
+                                                                   uint64_t cap, uint32_t *perm_ok,
+                                                                   OrderScan scan) {
+    grid_dep_wait();                     // the yield (and scan) pass has ended
+    extern __shared__ unsigned long long s_gpre[];      // SCAN: one entry per group
+    __shared__ uint32_t s_hist[kOrderRunWarps][kAzBins];
+    __shared__ uint16_t s_rank[kOrderRunWarps][kOrderRunCache];
+    const uint64_t total = order_prefix<SCAN, kOrderRunWarps>(em, scan, s_gpre);
+    const bool fits = total <= cap;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (fits) atomicOr(perm_ok, 1u);
+        if (SCAN) {
+            *scan.total = total;
+            scan.offsets[em.n_tracks] = total;
+        }
+    }
+    if (!SCAN && !fits) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t *const hist = s_hist[w];
+    uint16_t *const ranks = s_rank[w];
+    const int64_t n_warps = (int64_t)gridDim.x * kOrderRunWarps;
+    const int64_t run = (em.n_tracks + n_warps - 1) / n_warps;
+    const int64_t t0 = ((int64_t)blockIdx.x * kOrderRunWarps + w) * run;
+    const int64_t t1 = min(t0 + run, em.n_tracks);
+    if (t0 >= t1) return;
+    uint64_t off = 0;
+    if (SCAN) {
+        const int64_t g = t0 / kYieldThreads;
+        unsigned long long part = 0;
+        for (int64_t i = g * kYieldThreads + lane; i < t0; i += 32) part += scan.counts[i];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(kFull, part, o);
+        off = s_gpre[g] + part;
+    } else {
+        off = em.offsets[t0];
+    }
+    for (int64_t t = t0; t < t1; ++t) {                  // warp-uniform
+        const uint64_t n64 = SCAN ? (uint64_t)scan.counts[t] : em.offsets[t + 1] - off;
+        if (SCAN && lane == 0) scan.offsets[t] = off;
+        if (fits && n64 > kOrderMaxPhotons) {
+            if (lane == 0) atomicOr(perm_ok, 2u);
+        } else if (fits && n64 != 0) {
+            const uint32_t n = (uint32_t)n64;
+            const uint32_t id = em.tracks[t].id, ev = em.tracks[t].event;
+            hist[lane] = 0u;
+            __syncwarp();
+            const uint32_t kept = n < kOrderRunCache ? n : kOrderRunCache;
+            for (uint32_t j = lane; j < kept; j += 32) {
+                const uint32_t bin = philox10(0u, j, id, ev, em.key0, em.key1).y >> 27;
+                ranks[j] = (uint16_t)(bin << 11 | atomicAdd(&hist[bin], 1u));
+            }
+            __syncwarp();                // kept ranks stay below kOrderRunCache
+            for (uint32_t j = kOrderRunCache + lane; j < n; j += 32)
+                atomicAdd(&hist[philox10(0u, j, id, ev, em.key0, em.key1).y >> 27], 1u);
+            __syncwarp();
+            const uint32_t c = hist[lane];
+            uint32_t inc = c;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, inc, o);
+                if (lane >= o) inc += y;
+            }
+            __syncwarp();
+            // cursors: the bin's start for the photons with a kept rank, which are
+            // the first to be counted in it; those after them follow
+            hist[lane] = inc - c;
+            __syncwarp();
+            for (uint32_t j = lane; j < kept; j += 32) {
+                const uint32_t r = ranks[j];
+                perm[off + hist[r >> 11] + (r & 2047u)] = make_uint2(j, (uint32_t)t);
+            }
+            if (n > kOrderRunCache) {
+                // the kept photons of each bin counted again, then the rest behind them
+                __syncwarp();
+                for (uint32_t j = lane; j < kept; j += 32) atomicAdd(&hist[ranks[j] >> 11], 1u);
+                __syncwarp();
+                for (uint32_t j = kOrderRunCache + lane; j < n; j += 32) {
+                    const uint32_t bin = philox10(0u, j, id, ev, em.key0, em.key1).y >> 27;
+                    perm[off + atomicAdd(&hist[bin], 1u)] = make_uint2(j, (uint32_t)t);
+                }
+            }
+            __syncwarp();
+        }
+        off += n64;
+    }
+}
+
+static cudaError_t ensure_dyn_smem(const void *f, size_t bytes);
+
 cudaError_t launch_order(const EmitView &em, uint2 *perm, uint64_t cap, uint32_t *perm_ok,
                          int n_sm, cudaStream_t s, const OrderScan *scan) {
-    int64_t blocks = em.n_tracks;                       // one block per track
-    if (blocks < 1) blocks = 1;
-    const int64_t max_blocks = (int64_t)n_sm * 16;
-    if (blocks > max_blocks) blocks = max_blocks;
-    const bool early = em.n_tracks <= blocks;
-    if (scan) {
-        const int64_t groups = (em.n_tracks + kYieldThreads - 1) / kYieldThreads;
-        if (groups > kOrderScanGroups) return cudaErrorInvalidValue;
-        return launch_pdl(k_order<true>, (unsigned)blocks, 32 * kOrderWarps,
-                          sizeof(unsigned long long) * (size_t)groups, s, em, perm, cap, perm_ok,
-                          *scan, early);
+    const int64_t groups = (em.n_tracks + kYieldThreads - 1) / kYieldThreads;
+    if (scan && groups > kOrderScanGroups) return cudaErrorInvalidValue;
+    const size_t smem = scan ? sizeof(unsigned long long) * (size_t)groups : 0;
+    // a block per track up to four times the blocks that the SMs hold (3001
+    // tracks: 13 us, and 14 us as runs; 10^4: 26 and 24 us), else runs of tracks
+    if (em.n_tracks <= (int64_t)n_sm * kOrderBlocksPerSm) {
+        const unsigned blocks = em.n_tracks < 1 ? 1u : (unsigned)em.n_tracks;
+        if (scan)
+            return launch_pdl(k_order<true>, blocks, 32 * kOrderWarps, smem, s, em, perm, cap,
+                              perm_ok, *scan);
+        return launch_pdl(k_order<false>, blocks, 32 * kOrderWarps, smem, s, em, perm, cap, perm_ok,
+                          OrderScan{});
     }
-    return launch_pdl(k_order<false>, (unsigned)blocks, 32 * kOrderWarps, 0, s, em, perm, cap,
-                      perm_ok, OrderScan{}, early);
+    const unsigned blocks = (unsigned)n_sm * 6;
+    if (!scan)
+        return launch_pdl(k_order_run<false>, blocks, 32 * kOrderRunWarps, smem, s, em, perm, cap,
+                          perm_ok, OrderScan{});
+    // beside 33 KB of static shared memory
+    if (smem > 12 * 1024) {
+        const cudaError_t e = ensure_dyn_smem((const void *)k_order_run<true>, smem);
+        if (e != cudaSuccess) return e;
+    }
+    return launch_pdl(k_order_run<true>, blocks, 32 * kOrderRunWarps, smem, s, em, perm, cap,
+                      perm_ok, *scan);
 }
 
 // ============================================================== emission

@@ -84,3 +84,39 @@ def test_deferred_scan_matches_scan_pass_edge_cases(case):
     assert a[2] == b[2] == 1                       # both ordered
     for x, y in zip(a[3:], b[3:]):
         np.testing.assert_array_equal(x, y)
+
+
+@pytest.mark.parametrize("n_tracks", [9728, 9729, 20000])
+def test_ordering_of_many_tracks_leaves_the_photons_as_they_are(n_tracks):
+    """The azimuth order over a block per track (up to 64 tracks per SM) and
+    over runs of tracks, for photon counts at the edges of the kept ranks
+    (2048) and of the ordered tracks (16384), with the scan in the ordering
+    pass and ahead of it: fates and pixel counts as in index order."""
+    scene = W.rich1_scene(meshed=True)
+    tracks = W.pion_tracks(n_tracks, seed=8, p_min=3.0)
+    counts = np.tile([0, 1, 3, 33], n_tracks // 4 + 1)[:n_tracks]
+    edges = [2047, 2048, 2049, 5000, 16384]
+    counts[5:5 + len(edges)] = edges
+    counts[-1] = 700
+    for last in (16384, 16385):              # all ordered; one left in index order
+        counts[-3] = last
+        tracks.n_fixed = counts.astype(np.uint32)
+        n = int(counts.sum())
+        dt = rich.DeviceTracks(tracks)
+        seen = []
+        for order in ("index", "scan ahead", "scan inside"):
+            ctx = rich.Context(0)
+            ctx.init_geometry(scene)
+            if order != "index":
+                assert ctx.emit(dt, 0.0014, seed=2) == n     # sizes the order buffer
+            if order != "scan ahead":
+                ctx.emit(dt, 0.0014, seed=2, sync=False)
+            out = rich.TraceOutputs(n // 2, scene.pixels_per_event, 3, 1, n)
+            ctx.trace(out)
+            _, st = ctx.hits()
+            assert st["photon_order"] == (order != "index") and st["n_photons"] == n
+            seen.append((out.fate.cpu().numpy(), out.pixel_counts_numpy()))
+            ctx.close()
+        for fate, pixels in seen[1:]:
+            np.testing.assert_array_equal(fate, seen[0][0])
+            np.testing.assert_array_equal(pixels, seen[0][1])
