@@ -1076,6 +1076,9 @@ __device__ __noinline__ void nearest_tiles(const SmemScene &S, f3 o, f3 d, bool 
             const float vb = fmaf(vx, d.x, fmaf(vy, d.y, vz * d.z));
             if ((fmaf(-vb, vb, v2) > G.g2) | ((vb > 0.0f) & (v2 > G.g2))) continue;
         }
+        // the tile just left, alone on its sphere (10^6 photons of a point source: 104
+        // -> 96 us; with every tile tilted, 143 -> 134 us)
+        if (G.count == 1 && S.tiles()[G.first].prim == skip) continue;
         // w = o - C exactly (FP32 inputs)
         const ff wx = two_sum(o.x, -G.fcx), wy = two_sum(o.y, -G.fcy),
                  wz = two_sum(o.z, -G.fcz);
