@@ -299,16 +299,16 @@ typedef struct rich_trace_opts {
                                idle (1..32): the compaction interval (default
                                32, or 16 in scenes of rectangles alone)      */
     int32_t chunk;          /* photons a warp takes from the queue at a time
-                               (default 32, or 32..128 by what is left in
-                               scenes of rectangles alone)                   */
+                               (default 32..128, by what is left)            */
     int32_t wide_regs;      /* <= 256 threads: 0 caps the trace kernel at 64
                                registers (four blocks per SM), 1 uncapped;
                                257..896 threads: 1 caps it at 72 registers
                                (the 896-thread build), 0 at 64 (the
                                1024-thread build); > 896 threads: the
                                1024-thread build. Both builds of more than
-                               256 threads keep the photon state the BVH
-                               walk does not use in shared memory          */
+                               256 threads keep the photon state that the
+                               search for a surface does not use in shared
+                               memory                                       */
     int32_t bvh_smem_nodes; /* top BVH nodes (128 bytes each) staged in shared
                                memory per block by a TMA bulk copy
                                (-1: default, above 256 threads 256, or 16
@@ -484,10 +484,12 @@ RICH_API rich_status rich_set_timing(rich_ctx *ctx, int on);
 RICH_API rich_status rich_kernel_times(rich_ctx *ctx, rich_kernel_ms *out);
 
 /* Algorithmic work of one trace, counted by the counting build of the trace
- * kernel (the same traversal with per-thread tallies). From these tallies
- * and the sizes of the records the traversal reads (128-byte four-wide BVH
- * nodes, 48-byte triangles, 36-byte vertex normals) follow the FP32
- * operations and the bytes per photon that bound the kernel. */
+ * kernel. It finds the nearest triangle by the BVH walk (the general path),
+ * also where rich_trace uses the surfaces that the meshes lie on: the nodes
+ * and triangle tests are the walk's, the other tallies those of either path.
+ * From the tallies and the sizes of the records (128-byte four-wide BVH
+ * nodes, 48-byte triangles, 36-byte vertex normals, 8-byte grid cells) follow
+ * the FP32 operations and the bytes per photon that bound the kernel. */
 typedef struct rich_work {
     uint64_t photons;         /* photons that entered the trace            */
     uint64_t steps;           /* nearest-surface queries (bounce steps)    */
@@ -504,8 +506,8 @@ typedef struct rich_work {
 } rich_work;
 
 /* rich_trace of the last emission (fused photons; precision
- * RICH_PREC_REFINE64; more than 256 block_threads -- the 80- and 64-register
- * shapes, which have a counting build) through the counting build, then
+ * RICH_PREC_REFINE64; more than 256 block_threads -- the 72- and 64-register
+ * builds, which have a counting form) through the counting build, then
  * the counters (as rich_hits) and the tallies into *work (host).
  * Synchronous; slower than rich_trace (for measurement only). Results
  * (hits, fates, histograms) are those of rich_trace. RICH_ERR_ARG for

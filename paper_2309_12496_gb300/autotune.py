@@ -2,8 +2,8 @@
 
 The persistent trace kernel's speed depends on the block shape (256 threads
 capped at 64 registers, four blocks per SM; 256 uncapped; 512, 768 or 896
-threads capped at 72 registers; 512 or 1024 threads capped at 64), on how many top BVH nodes each block stages in shared
-memory, on the compaction interval (refill a warp once `refill_min` lanes
+threads capped at 72 registers; 512 or 1024 threads capped at 64), on how
+many top BVH nodes each block stages in shared memory, on the compaction interval (refill a warp once `refill_min` lanes
 are idle) and on the photons a warp takes from the queue at a time. Which
 combination wins depends on the scene and on the number of photons (a small
 batch is dominated by the tail of the persistent grid). `tune` times every
@@ -43,6 +43,9 @@ def candidates(n_triangles: int):
             for refill in (24, 32):
                 out.append(dict(block_threads=threads, blocks_per_sm=0, bvh_smem_nodes=n,
                                 refill_min=refill, chunk=32, wide_regs=1))
+    # the library's own defaults (chunks by the photons left)
+    out.append(dict(block_threads=1024, blocks_per_sm=0, bvh_smem_nodes=-1, refill_min=0,
+                    chunk=0))
     return out
 
 

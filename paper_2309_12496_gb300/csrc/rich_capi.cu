@@ -548,10 +548,9 @@ int staged_nodes(const rich_ctx *ctx, int opt, int threads, bool proxies) {
 
 // A scene of rectangles alone: a photon's step costs the same wherever it goes,
 // so a warp refills when half its lanes are idle (photons make 1 to 8 bounces in
-// a mirror box) and takes up to 128 photons at a time: scintillator box, 4e6
-// photons, 792 us with 32 idle lanes and chunks of 32, 587 us with 16 and 32, 565 us
-// with 16 and 128, 546 us with 16 and a share of the photons left of 32 to 128 (12
-// and 20 idle lanes: 544 and 561 us); water tank, 6.6e6 photons, 317 -> 258 us.
+// a mirror box): scintillator box, 4e6 photons, chunks of 32, 792 -> 587 us (with
+// chunks of 32 to 128: 12, 16 and 20 idle lanes 544, 546 and 561 us); water tank,
+// 6.6e6 photons, 317 -> 258 us with both.
 // Scenes with curved or meshed mirrors refill idle warps only, which keeps a
 // warp's photons on the same mirror (RICH1, 10^4 tracks: 32 idle lanes 579 us, 24
 // 612 us, 16 661 us; analytic 585, 634, 692 us).
@@ -1142,7 +1141,14 @@ static rich_status trace_impl(rich_ctx *ctx, const rich_photons *in, const rich_
     p.t_min = o->t_min;
     p.refill_min = refill;
     p.chunk = chunk;
-    if (!o->chunk && flat_scene(ctx)) {
+    // By default a warp takes a share of the photons left, 32 to 128 at a time: all
+    // 128 while more than 2^21 are left, 32 below 2^20. Fewer trips to the queue and
+    // one track lookup per 128 photons, and small chunks at the end, so that the warps
+    // end together. Trace with chunks of 32 -> here: scintillator box (4e6 photons) 587
+    // -> 546 us, 10^4 RICH1 tracks 417 -> 413 us, 10^5 RICH2 tracks 3248 -> 3210 us;
+    // below 2^20 photons nothing changes. Up to 256: box 514 -> 510 us, 413 and 3201 us;
+    // up to 256 with twice the share: 525, 432 and 3215 us.
+    if (!o->chunk) {
         p.chunk_max = 128;
         p.chunk_shift = 14;
     }
