@@ -1,6 +1,6 @@
 // rich_kernels.cu -- sm_103a kernels of the Cherenkov photon propagator.
 //
-//   k_yield        one thread per track, double-word FP32: beta, Cherenkov angle
+//   k_yield        four lanes per track, double-word FP32: beta, Cherenkov angle
 //                  (cos theta = 1/(n beta), Sec. 3), Frank-Tamm mean and the
 //                  keyed Poisson photon count; block sums of the counts.
 //   k_offsets      exclusive scan of the counts into photon offsets
@@ -8,13 +8,20 @@
 //                  sums, then an in-block warp-shuffle scan).
 //   k_materialize  optional: photons written out as a structure of arrays
 //                  (the "vector of positions and momenta" of Sec. 4.2).
+//   k_order        optional: azimuth order of each track's photons, so that a
+//                  warp's photons go to the same mirror.
 //   k_trace        persistent propagation kernel: warps take chunks of
 //                  photons from an atomic queue, generate them in registers
 //                  (fused emission), trace them bounce by bounce and refill
 //                  idle lanes with new photons (warp-level compaction by
 //                  ballot/popc), apply reflectivity and quantum-efficiency
 //                  accept/reject in flight (Sec. 4.3 and Sec. 6), append
-//                  hits with warp-aggregated atomics and bin them.
+//                  hits with warp-aggregated atomics and bin them. Meshes on
+//                  few spheres or planes are searched through those surfaces
+//                  and a grid of triangle lists, other meshes through a BVH.
+//   k_refine       the detected photons' paths replayed in double-word FP32:
+//                  positions, times, reflection moments and event sums.
+//   k_adjoint      reverse pass of ring moments to the tracks' parameters.
 #include <climits>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -34,10 +41,10 @@ namespace rich {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
 
-// The photon state the BVH walk does not use (wavelength, the QE and
-// reflectivity words, the keys, indices and counters) kept in per-thread
-// shared memory instead of registers, by the two shapes of one block per SM
-// (more than 256 threads).
+// The photon state the search for the nearest surface does not use (wavelength,
+// the QE and reflectivity words, the keys, indices and counters) kept in
+// per-thread shared memory instead of registers, by the two builds of one block
+// per SM (more than 256 threads).
 #ifndef RICH_COLD_SMEM
 #define RICH_COLD_SMEM 1
 #endif
@@ -1952,13 +1959,13 @@ __device__ __forceinline__ uint32_t cold_refl_word(const ColdState &c, int k,
     return k == 0 ? w.x : (k == 1 ? w.y : (k == 2 ? w.z : w.w));
 }
 
-// PROXY: the scene's triangles all lie on surface proxies (the counting build
-// always walks the BVH: its tallies are the walk's).
-// The same out of line, for the trace.
+// find_track_warp out of line, for the trace.
 __device__ __noinline__ int64_t find_track(const EmitView &em, uint64_t g, int lane) {
     return find_track_warp(em, g, lane);
 }
 
+// PROXY: the scene's triangles all lie on surface proxies (the counting build
+// always walks the BVH: its tallies are the walk's).
 template <bool EXT, bool REFINE, int THREADS, int MINB, bool PROXY, bool COUNT = false>
 __global__ void __launch_bounds__(THREADS, MINB)
 k_trace(TraceArgs A) {
@@ -2105,8 +2112,8 @@ k_trace(TraceArgs A) {
     bool alive = false;
     int path[RICH_MAX_BOUNCES];
     WorkTally tally{};
-    // the shapes of one block per SM (896 threads at 72 registers, 1024 at
-    // 64) keep the cold photon state in shared memory (there it removes the
+    // the builds of one block per SM (1024 threads at 64 registers, 896 at
+    // 72) keep the cold photon state in shared memory (there it removes the
     // bounce loop's spills); the 256-thread shapes keep it in registers
     constexpr bool kColdOn = RICH_COLD_SMEM && THREADS > 256;
     const ColdState cold{cold_off + (uint32_t)threadIdx.x * (uint32_t)(sizeof(uint32_t) * kColdWords)};
