@@ -84,10 +84,17 @@ WORK_COST = {
     # per detected photon: plane coordinates (3 subtractions, 2 dots), QE
     # lookup, pixel (2 products)
     "detected": {"fp32": 3 + 10 + 2 + 2, "minmax": 0, "mufu": 0},
+    # crossing of a sphere that meshed mirrors lie on, and its grid cell: the
+    # origin from the centre (3 subtractions), its part along the ray and
+    # across it (a dot, 3 FMAs), r^2 less its square (a dot, a subtraction),
+    # the root and the distance (add), the point (3 FMAs) and the two cell
+    # coordinates (2 dots and 2 FMAs); min/max: the distance within
+    # [t_min, the nearest so far]
+    "crossing": {"fp32": 3 + 5 + 6 + 5 + 1 + 1 + 6 + 10 + 4, "minmax": 2, "mufu": 1},
 }
 # bytes each tallied event reads or writes outside shared memory
 BYTES = {"node": 128, "tri": 48, "normal": 36, "track": 64, "perm": 8, "hit": 40,
-         "refine_rec": 40}
+         "refine_rec": 40, "cell": 8}
 
 
 def kernel_source_hash():
@@ -129,6 +136,22 @@ def work_per_photon(w):
     per["bytes"] = outside + per["smem_bytes"]
     per["bytes_outside_smem"] = outside
     per["events_per_photon"] = {e: ev[e] / n for e in ev}
+    return per
+
+
+def least_work_per_photon(w):
+    """The same for a search that goes straight to the triangle hit, as the
+    timed kernel does where meshes lie on few spheres or planes: per direction
+    change one crossing, one grid cell and one triangle, and no BVH node. What
+    it does beyond that (crossings that hit nothing, cells with two triangles,
+    the bounding-sphere tests) is not counted: a lower bound of the work."""
+    per = work_per_photon(dict(w, nodes_smem=0, nodes_global=0, tri_tests=w["turns"]))
+    n = max(1, w["photons"])
+    for k in ("fp32", "minmax", "mufu"):
+        per[k] += w["turns"] * WORK_COST["crossing"][k] / n
+    for k in ("bytes", "bytes_outside_smem"):
+        per[k] += w["turns"] * BYTES["cell"] / n
+    per["events_per_photon"]["crossing"] = w["turns"] / n
     return per
 
 
@@ -427,20 +450,20 @@ def roofline(ctx, dt, out, seeds, photons, flush, knobs, prec, peaks, clk):
 
     Its own duration comes from the library's kernel timing (events around
     k_trace on the context's stream) over the same seeds as the timed steps,
-    L2 flushed before each. Its work per photon comes from the counting
-    build (rich_trace_work) on the first seed: FP32 operations and the bytes
-    of the BVH nodes, triangles, normals and records its traversal reads and
-    writes (WORK_COST, BYTES), wherever the kernel keeps them. The two
-    bounds are those of the scope: FP32 work over the measured FP32 FMA
-    rate, and bytes per photon over the measured L2 read bandwidth; `bound`
-    is the slower, and `frac` the kernel's achieved rate over that bound's
-    peak. The kernel keeps the top BVH levels in shared memory, which is
-    how it could run faster than the L2 bound. Beside them: the bound with
-    only the bytes read from outside shared memory, the min/max (ALU) and
-    special-function rates against their measured peaks, and, from the
-    committed ncu capture when it was taken from these sources, warp
-    instructions and the DRAM and L2 bytes per photon that the kernel
-    actually moved."""
+    L2 flushed before each. Its work per photon follows from the tallies of
+    the counting build (rich_trace_work) on the first seed. The timed kernel
+    finds RICH1's mirrors through the spheres and planes they lie on, so the
+    work is that of a direct search (least_work_per_photon): FP32 operations
+    and the bytes of the cells, triangles, normals and records. The two
+    bounds are FP32 work over the measured FP32 FMA rate, and bytes per photon
+    over the measured L2 read bandwidth; `bound` is the slower, and `frac` the
+    kernel's achieved rate over that bound's peak. Beside them: the min/max
+    (ALU) and special-function rates against their measured peaks, `bvh_walk`,
+    the bounds of the walk that the counting build tallies (the kernel's path
+    on meshes of any other form; a rate above 1 of those says that the direct
+    search leaves that work out), and, from the committed ncu capture when it
+    was taken from these sources, warp instructions and the DRAM and L2 bytes
+    per photon that the kernel actually moved."""
     import torch
     from paper_2309_12496_gb300 import rich
     stream = torch.cuda.current_stream()
@@ -466,7 +489,8 @@ def roofline(ctx, dt, out, seeds, photons, flush, knobs, prec, peaks, clk):
     out.clear()
     tally = ctx.trace_work(out, **{k: v for k, v in wk.items()})
     torch.cuda.synchronize()
-    w = work_per_photon(tally)
+    w = least_work_per_photon(tally)
+    walk = work_per_photon(tally)
     rate = ph_step / t_trace                              # photons/s in k_trace
     fp32 = {"per_photon": w["fp32"], "achieved": w["fp32"] * rate / 1e12,
             "peak": peaks["fp32_fma_flops"] / 1e12, "unit": "TFLOP/s"}
@@ -492,6 +516,10 @@ def roofline(ctx, dt, out, seeds, photons, flush, knobs, prec, peaks, clk):
     for b in (fp32, l2, l2_out, alu, xu, hbm):
         b["frac"] = b["achieved"] / b["peak"]
         b["photons_per_s_bound"] = rate / b["frac"]
+    bvh_walk = {"fp32": {"per_photon": walk["fp32"],
+                         "frac": walk["fp32"] * rate / peaks["fp32_fma_flops"]},
+                "l2": {"per_photon": walk["bytes"],
+                       "frac": walk["bytes"] * rate / peaks["l2_read_bytes"]}}
     bound = "l2" if l2["frac"] >= fp32["frac"] else "fp32"
     main = l2 if bound == "l2" else fp32
     prof = load_profile()
@@ -515,6 +543,9 @@ def roofline(ctx, dt, out, seeds, photons, flush, knobs, prec, peaks, clk):
             "peak_source": "measured by rich_measure_peaks in this run (of measured)",
             "bounds": {"fp32": fp32, "l2": l2, "l2_outside_smem": l2_out, "alu_minmax": alu,
                        "mufu": xu, "hbm": hbm},
+            "work": "direct search: one crossing, cell and triangle per direction change "
+                    "(lower bound of the timed kernel's work)",
+            "bvh_walk": bvh_walk,
             "smem_bytes_per_photon": w["smem_bytes"],
             "events_per_photon": w["events_per_photon"],
             "work_tally": tally, "peaks": peaks, "issue": issue,
