@@ -2180,7 +2180,7 @@ k_trace(TraceArgs A) {
                     }
                     // a warp's first chunk is its place in the grid, over the SMs
                     // first: with no atomic, the warps' start is not serialised on
-                    // the counter (4864 of them; 5 x 10^4 photons 26 -> 22.5 us, RICH1,
+                    // the counter (4864 of them; 1.6 x 10^4 photons 26 -> 22.5 us, RICH1,
                     // 10^4 tracks, 415 -> 411 us, RICH2 3223 -> 3191 us; over the warps
                     // of an SM first: 28, 411 and 3191 us)
                     if (pool_end == 0) {
