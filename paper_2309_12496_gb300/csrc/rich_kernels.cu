@@ -2638,6 +2638,11 @@ k_refine(SceneView sc, EmitView em, ExtView ext, TraceParams P, Counters *ctr) {
         }
     }
     if (own) {
+        // lane 4 k + q keeps sum q of key k, so that the FP64 conversions and the
+        // atomics of all keys are one instruction each (one lane's chain of them
+        // before: 1000 RICH1 tracks 18.4 -> 16.4 us, the call 88.2 -> 86.3 us)
+        ff mine = ffv(0.0f);
+        uint32_t got = 0u;
         for (int k = 0; k < n_keys; ++k) {
             const uint32_t n = __reduce_add_sync(kFull, s_own_n[k][threadIdx.x]);
             if (n == 0) continue;        // uniform in the warp
@@ -2648,11 +2653,15 @@ k_refine(SceneView sc, EmitView em, ExtView ext, TraceParams P, Counters *ctr) {
             for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
                 for (int q = 0; q < 3; ++q) a[q] = ff_add(a[q], shfl_xor_ff(a[q], o));
-            if (lane == 0) {
-                atomicAdd(s_es + 4 * k, (double)n);
-                for (int q = 0; q < 3; ++q) atomicAdd(s_es + 4 * k + 1 + q, ff_to_double(a[q]));
+            if ((lane >> 2) == k) {
+                got = n;
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+                    if ((lane & 3) == q + 1) mine = a[q];
             }
         }
+        if (got != 0u)
+            atomicAdd(s_es + lane, (lane & 3) == 0 ? (double)got : ff_to_double(mine));
     }
     __syncthreads();
     if (s_es) es_table_flush(sc, P, s_es);

@@ -1,0 +1,61 @@
+"""Event sums of the refined path against the hit list it belongs to (marked
+gpu): per (event, plane) key the count and the sums of u, v and lambda, at the
+key counts where the summing changes (per thread up to 4 keys, a block's table
+up to 64, global sums above), with events that have no hits and warps that have
+none."""
+import numpy as np
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2309_12496_gb300 import build, rich  # noqa: E402
+from paper_2309_12496_gb300 import workloads as W  # noqa: E402
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    build.build()
+
+
+# keys = events x planes: 1, 3, 4, 5, 6, 63, 64, 65, 66
+@pytest.mark.parametrize("name,n_events", [("point", 1), ("rich1", 1), ("point", 4),
+                                           ("point", 5), ("rich1", 2), ("rich1", 21),
+                                           ("point", 64), ("point", 65), ("rich1", 22)])
+@pytest.mark.parametrize("photons", [1, 33, 20_000])
+def test_event_sums_are_those_of_the_hits(name, n_events, photons):
+    scene = W.point_source_scene() if name == "point" else W.rich1_scene(meshed=True)
+    rng = np.random.default_rng(photons + n_events)
+    n = photons
+    d = np.stack([rng.uniform(-0.2, 0.2, n), rng.uniform(-0.2, 0.2, n), np.ones(n)], 1)
+    d = (d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32)
+    pb = rich.PhotonBuffers.from_arrays(**{
+        "x": rng.uniform(-20, 20, n), "y": rng.uniform(-20, 20, n), "z": rng.uniform(0, 50, n),
+        "dx": d[:, 0], "dy": d[:, 1], "dz": d[:, 2], "lambda": rng.uniform(300, 500, n),
+        # the last event of several gets no photon
+        "event": rng.integers(0, max(1, n_events - 1), n),
+        "track": np.arange(n), "photon": np.zeros(n)})
+    ctx = rich.Context(0)
+    ctx.init_geometry(scene)
+    planes = len(scene.planes)
+    assert planes == (1 if name == "point" else 3)
+    out = rich.TraceOutputs(n, scene.pixels_per_event, planes, n_events, n)
+    ctx.trace(out, photons=pb, seed=5)
+    n_hits, _ = ctx.hits()
+    h = out.hits_numpy(n_hits)
+    sums = out.event_sums_numpy()
+    ctx.close()
+    assert n_hits == len(h) and (photons < 1000 or n_hits > 500)
+    for e in range(n_events):
+        for p in range(planes):
+            g = h[(h["event"] == e) & (h["plane"] == p)]
+            assert sums[e, p, 0] == len(g)
+            for k, f in ((1, "u"), (2, "v"), (3, "lambda")):
+                x = g[f].astype(np.float64)
+                # double-word additions, 2^-44 each of the partial sum; a term
+                # passes at most 3 (per thread) + 5 (warp) of them, then at most 625
+                # FP64 additions (one per warp with hits): 8 + 1.3 of 2^-44
+                assert abs(sums[e, p, k] - x.sum()) <= 16 * 2.0 ** -44 * np.abs(x).sum()
