@@ -96,6 +96,10 @@ struct alignas(16) DevNode { // 128 B: boxes of up to four children (by axis) + 
 
 // One sphere or plane that a set of meshed surfaces follows, and the grid over
 // its projection along the axis, in units of its cells (rich_proxy.h).
+// A step tests every proxy's bounding sphere, so their number is bounded: trace of
+// 10^4 RICH1 tracks with 4, 6 and 8 proxies (tiles and halves of the flat mirrors
+// turned by 2 to 8 mrad) 409, 411 and 434 us, by the BVH 897, 895 and 923 us; more
+// were not measured, and a scene with more walks the BVH.
 #define RICH_MAX_PROXIES 8
 struct alignas(16) DevProxy {  // 128 B, read as 16-byte words
     float cx, cy, cz, dt;      // centre, or a point of the plane; bound of the along-ray
