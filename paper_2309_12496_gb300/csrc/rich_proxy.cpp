@@ -160,6 +160,23 @@ bool fit_sphere(const std::vector<DevTri> &T, const std::vector<int> &sel, Fit &
     return f.r > 0.0;
 }
 
+// Longest way along a ray from its crossing of the sphere or plane, at a cosine of
+// at least kProxyCosMin, to a point within the shell (and the rounding error E). To
+// a plane's it is depth / cosine. Inside a sphere the ray flattens on its way: from
+// radius r at cosine c to radius r - s it is r c - sqrt(r^2 c^2 - 2 r s + s^2), longer
+// than s / c by some s^2 (1 - c^2) / (2 r c^3) (outwards it is shorter than s / c). 0:
+// a ray at the limit does not come as deep as s, and no such bound holds. The squared
+// cosine of a crossing that passes the FP32 test may be below the limit by E / r
+// (16 u W / r from q2 and 4 u from r^2, W >= r).
+double shell_reach(const Fit &f, double E) {
+    const double s = f.shell + E;
+    if (!(f.r > 0.0)) return s / kProxyCosMin;
+    const double c2 = (double)kProxyCosMin * kProxyCosMin - E / f.r;
+    const double in2 = f.r * f.r * c2 - 2.0 * f.r * s + s * s;
+    if (!(c2 > 0.0 && in2 > 0.0 && s < f.r)) return 0.0;
+    return f.r * std::sqrt(c2) - std::sqrt(in2);
+}
+
 // Grid and device record of one fit; false when the margin does not suit it.
 bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, ProxyResult &out) {
     const bool sphere = f.r > 0.0;
@@ -215,7 +232,9 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     // the scene's box), and the margins
     const double W = o_max(extent) + len(f.c), W_g = o_max(extent) + len(g);
     const double E = 32.0 * kUnit * W;
-    const double margin = (f.shell + E) / kProxyCosMin + E;
+    const double reach = shell_reach(f, E);
+    if (!(reach > 0.0)) return false;
+    const double margin = reach + E;
     const double tri_size = std::sqrt(area / (double)f.tris.size());
     double size = std::max(kCellScale * tri_size, 4.0 * margin);
     const double wx = hi[0] - lo[0] + 4.0 * margin, wy = hi[1] - lo[1] + 4.0 * margin;
@@ -237,9 +256,9 @@ bool make_proxy(const std::vector<DevTri> &T, const Fit &f, double extent, Proxy
     DevProxy P;
     std::memset(&P, 0, sizeof P);
     P.cx = (float)f.c[0]; P.cy = (float)f.c[1]; P.cz = (float)f.c[2]; P.r = (float)f.r;
-    P.dt = (float)((f.shell + E) / kProxyCosMin + E);
+    P.dt = (float)margin;
     P.ax = (float)axis[0]; P.ay = (float)axis[1]; P.az = (float)axis[2];
-    P.z_min = (float)(0.5 * lo[2]);
+    P.z_min = (float)std::min(0.5 * lo[2], lo[2] - margin);
     P.e1x = (float)f1[0]; P.e1y = (float)f1[1]; P.e1z = (float)f1[2]; P.x0 = x0;
     P.e2x = (float)f2[0]; P.e2y = (float)f2[1]; P.e2z = (float)f2[2]; P.y0 = y0;
     P.fnx = (float)nx; P.fny = (float)ny; P.nx = nx;

@@ -37,8 +37,10 @@ namespace rich {
 // the surface (the roundings of w, of the dots and, after the Newton step on
 // |p| = r, of |p|^2 - r^2), by 8 u W / c along the ray for an angle of
 // incidence with cosine c >= kProxyCosMin, and a facet's point lies within
-// `shell` of the surface; the cells' margin holds (shell + E) / kProxyCosMin + E
-// with E = 32 u W. A crossing is found by selects instead of branches: a
+// `shell` of the surface. The cells' margin, which is also DevProxy::dt, holds the
+// longest way of such a ray through shell + E, E = 32 u W, and E once more: for a
+// plane (shell + E) / kProxyCosMin + E, for a sphere somewhat more, as a ray that
+// enters it flattens (shell_reach in rich_proxy.cpp). A crossing is found by selects instead of branches: a
 // warp's rays mostly take the same surfaces, and control flow was a fifth of the
 // trace's instructions.
 constexpr float kProxyCosMin = 0.25f;

@@ -19,11 +19,12 @@ from paper_2309_12496_gb300 import workloads as W
 WRAP = r"""
 #include "rich_bvh.h"
 #include "rich_proxy.h"
+#include <algorithm>
 #include <cstring>
 using namespace rich;
 extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, double extent, int64_t nr,
                           const float *o, const float *d, const int32_t *target, float t_max,
-                          uint8_t *out, double *listed) {
+                          uint8_t *out, double *listed, const double *t_hit, double *reach) {
     BvhResult b;
     std::string err;
     if (!build_bvh(v, surf, nt, b, err)) return -1;
@@ -49,7 +50,7 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
         for (size_t k = 0; k < R.proxies.size(); ++k) {
             const DevProxy &P = R.proxies[k];
             int cell[2] = {-1, -1};
-            float t, b2, h2;
+            float t, t_in = 0.0f, b2, h2;
             bool sure, entering = false;
             if (proxy_misses(P, O[0], O[1], O[2], D[0], D[1], D[2], t_max)) continue;
             if ((int)k < R.n_planes) {
@@ -59,9 +60,14 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
                                        entering, b2, h2);
                 if (entering)
                     cell[1] = proxy_sphere_side(P, O[0] - P.cx, O[1] - P.cy, O[2] - P.cz, D[0], D[1],
-                                                D[2], b2, h2, -1.0f, 1e-3f, t_max, t, true);
+                                                D[2], b2, h2, -1.0f, 1e-3f, t_max, t_in, true);
             }
             if (!sure) out[i] |= 2;
+            if (t_hit && sure) {
+                double far = std::fabs(t - t_hit[i]);
+                if (entering) far = std::min(far, std::fabs(t_in - t_hit[i]));
+                *reach = std::max(*reach, far / P.dt);
+            }
             for (int c : cell) {
                 if (c < 0) continue;
                 const DevProxyCell &L = R.cells[k][(size_t)(c - P.first_cell)];
@@ -75,6 +81,39 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
     }
     *listed = nr ? tests / (double)nr : 0.0;
     return (int)R.proxies.size();
+}
+// The nearest triangle ahead of each ray in FP64, or -1: none, or met within 1e-3
+// of an edge (where FP32 may see its neighbour).
+extern "C" void nearest_tri(int64_t nt, const float *v, int64_t nr, const float *o, const float *d,
+                            int32_t *target, double *t_hit) {
+    for (int64_t i = 0; i < nr; ++i) {
+        const double O[3] = {o[3 * i], o[3 * i + 1], o[3 * i + 2]};
+        const double D[3] = {d[3 * i], d[3 * i + 1], d[3 * i + 2]};
+        double best = 1e300;
+        target[i] = -1;
+        for (int64_t k = 0; k < nt; ++k) {
+            double a[3], e1[3], e2[3];
+            for (int c = 0; c < 3; ++c) {
+                a[c] = O[c] - v[9 * k + c];
+                e1[c] = (double)v[9 * k + 3 + c] - v[9 * k + c];
+                e2[c] = (double)v[9 * k + 6 + c] - v[9 * k + c];
+            }
+            const double p[3] = {D[1] * e2[2] - D[2] * e2[1], D[2] * e2[0] - D[0] * e2[2],
+                                 D[0] * e2[1] - D[1] * e2[0]};
+            const double q[3] = {a[1] * e1[2] - a[2] * e1[1], a[2] * e1[0] - a[0] * e1[2],
+                                 a[0] * e1[1] - a[1] * e1[0]};
+            const double det = e1[0] * p[0] + e1[1] * p[1] + e1[2] * p[2];
+            if (det == 0.0) continue;
+            const double b1 = (a[0] * p[0] + a[1] * p[1] + a[2] * p[2]) / det;
+            const double b2 = (D[0] * q[0] + D[1] * q[1] + D[2] * q[2]) / det;
+            const double t = (e2[0] * q[0] + e2[1] * q[1] + e2[2] * q[2]) / det;
+            const double in = std::min(std::min(b1, b2), 1.0 - b1 - b2);
+            if (in < -1e-3 || t < 1e-2 || t >= best) continue;
+            best = t;
+            t_hit[i] = t;
+            target[i] = in >= 1e-3 ? (int32_t)k : -1;
+        }
+    }
 }
 """
 
@@ -118,6 +157,20 @@ SCENES = {
 }
 
 
+def _find(lib, v, surf, extent, o, d, k, t_hit=None):
+    """proxy_find on rays (o, d) with target triangles k, met at t_hit: proxies,
+    flags, and the largest distance along a ray from its crossing to the
+    triangle, as a share of the bound (one proxy)."""
+    out = np.zeros(len(o), np.uint8)
+    listed, reach = C.c_double(), C.c_double()
+    p = [None if a is None else a.ctypes.data_as(C.c_void_p)
+         for a in (v, None if surf is None else np.ascontiguousarray(surf, np.int32),
+                   o, d, k, out, t_hit)]
+    n = lib.proxy_find(C.c_int64(len(v)), p[0], p[1], C.c_double(extent), C.c_int64(len(o)), p[2],
+                       p[3], p[4], C.c_float(3e38), p[5], C.byref(listed), p[6], C.byref(reach))
+    return n, out, reach.value
+
+
 def _rays(v, n, rng, cos_min, dist):
     """Rays at points of random triangles: inside, on edges, at corners."""
     k = rng.integers(0, len(v), n)
@@ -146,19 +199,71 @@ def test_a_ray_finds_the_triangle_it_meets_or_goes_to_the_bvh(lib, name, cos_min
     v = np.ascontiguousarray(v, np.float32)
     n = 60000
     k, o, d = _rays(v, n, np.random.default_rng(len(v)), cos_min, dist)
-    out = np.zeros(n, np.uint8)
-    listed = C.c_double()
-    s = None if surf is None else np.ascontiguousarray(surf, np.int32)
-    n_proxies = lib.proxy_find(C.c_int64(len(v)), v.ctypes.data_as(C.c_void_p),
-                               None if s is None else s.ctypes.data_as(C.c_void_p),
-                               C.c_double(float(np.abs(v).max())), C.c_int64(n),
-                               o.ctypes.data_as(C.c_void_p), d.ctypes.data_as(C.c_void_p),
-                               k.ctypes.data_as(C.c_void_p), C.c_float(3e38),
-                               out.ctypes.data_as(C.c_void_p), C.byref(listed))
+    n_proxies, out, _ = _find(lib, v, surf, float(np.abs(v).max()), o, d, k)
     assert n_proxies == {"rich1": 4, "rich2": 5}.get(name, 1)
     assert np.all(out != 0), (int((out == 0).sum()), np.flatnonzero(out == 0)[:5])
     if cos_min > 0.25 and dist < 5000:
         assert (out & 1).mean() > 0.5            # most by their cells
+
+
+# (radius, half width, cells): facet edges of 0.1 to 0.4 of the radius, the
+# builder's limit among them, and whether they get a proxy
+COARSE = {"r500_10": (500.0, 100.0, 4, 1), "r2700_18": (2700.0, 500.0, 2, 1),
+          "r500_20": (500.0, 150.0, 3, 1), "r1000_25": (1000.0, 250.0, 2, 1),
+          "r500_27": (500.0, 200.0, 3, 1), "r500_30": (500.0, 150.0, 2, 1),
+          "r1000_30": (1000.0, 300.0, 2, 1), "r2700_30": (2700.0, 800.0, 2, 1),
+          "r500_40": (500.0, 200.0, 2, 0)}
+
+
+@pytest.mark.parametrize("name", sorted(COARSE))
+def test_coarse_facets_are_found_at_the_steepest_crossings(lib, name):
+    """The shell between a sphere and its facets is thick here against the
+    radius, and a ray near the cosine limit runs through it for longer than its
+    thickness over the cosine. Rays at the deepest points of the facets
+    (the middles of edges, a little inside) that cross the proxy's sphere at
+    cosines 0.24 to 0.3, checked on the triangle that they meet first and on the
+    distance from the crossing to it."""
+    radius, half, cells, n_expected = COARSE[name]
+    v, surf = _patch(radius, half, cells, 1.0)
+    n = 1_000_000
+    rng = np.random.default_rng(int(radius + half + cells))
+    k = rng.integers(0, len(v), n)
+    e = rng.integers(0, 3, n)
+    b = np.zeros((n, 3))
+    b[np.arange(n), e] = rng.uniform(0.35, 0.65, n)
+    b[np.arange(n), (e + 1) % 3] = 1.0 - b[np.arange(n), e]
+    b[np.arange(n), (e + 2) % 3] = rng.uniform(0.001, 0.1, n)
+    b /= b.sum(1, keepdims=True)
+    t = v[k].astype(np.float64)
+    p = np.einsum("ij,ijk->ik", b, t)
+    # the proxy's sphere: the centre, and a radius in the middle of the facets'
+    q = v.reshape(-1, 3).astype(np.float64)
+    x = np.linalg.lstsq(np.c_[2 * q, np.ones(len(q))], (q * q).sum(1), rcond=None)[0][:3]
+    g = np.cross(t[:, 1] - t[:, 0], t[:, 2] - t[:, 0])
+    inner = np.abs(((t[:, 0] - x) * g).sum(1) / np.linalg.norm(g, axis=1)).min()
+    r = 0.5 * (inner + np.linalg.norm(q - x, axis=1).max())
+    nrm = p - x
+    rho = np.linalg.norm(nrm, axis=1)
+    nrm /= rho[:, None]
+    s2 = (1.0 - rng.uniform(0.24, 0.3, n) ** 2) * (r / rho) ** 2
+    c = np.sqrt(np.maximum(0.0, 1.0 - s2)) * rng.choice([-1.0, 1.0], n)
+    side = rng.standard_normal((n, 3))
+    side -= (side * nrm).sum(1, keepdims=True) * nrm
+    side /= np.linalg.norm(side, axis=1, keepdims=True)
+    d = (c[:, None] * nrm + np.sqrt(1 - c * c)[:, None] * side).astype(np.float32)
+    o = (p - d * rng.uniform(0.2, 1.0, (n, 1)) * radius).astype(np.float32)
+    k = np.zeros(n, np.int32)
+    t_hit = np.zeros(n)
+    lib.nearest_tri(C.c_int64(len(v)), v.ctypes.data_as(C.c_void_p), C.c_int64(n),
+                    *(a.ctypes.data_as(C.c_void_p) for a in (o, d, k, t_hit)))
+    on = k >= 0
+    assert on.mean() > 0.3
+    n_proxies, out, reach = _find(lib, v, surf, float(np.abs(v).max()) + radius, o[on], d[on],
+                                  k[on], t_hit[on])
+    assert n_proxies == n_expected
+    if n_proxies:
+        assert np.all(out != 0), (int((out == 0).sum()), len(out))
+        assert 0.1 < reach <= 1.0
 
 
 def test_meshes_off_any_sphere_or_plane_use_the_bvh(lib):
@@ -176,8 +281,5 @@ def test_meshes_off_any_sphere_or_plane_use_the_bvh(lib):
     surfs = (None, None, np.repeat(np.arange(9, dtype=np.int32), len(v)))
     for m, s in zip((bent, ball, many), surfs):
         m = np.ascontiguousarray(m, np.float32)
-        listed = C.c_double()
-        assert lib.proxy_find(C.c_int64(len(m)), m.ctypes.data_as(C.c_void_p),
-                              None if s is None else s.ctypes.data_as(C.c_void_p),
-                              C.c_double(1000.0), C.c_int64(0), None, None, None, C.c_float(1.0),
-                              None, C.byref(listed)) == 0
+        none = np.zeros((0, 3), np.float32)
+        assert _find(lib, m, s, 1000.0, none, none, np.zeros(0, np.int32))[0] == 0
