@@ -777,9 +777,8 @@ def _ring_chi2_function():
 
     class _RingChi2(torch.autograd.Function):
         @staticmethod
-        def forward(fctx, th, ctx, tracks, targets, outputs, sigma, seed):
-            loss, grad, used = ctx.trace_grad(tracks, th.detach().cpu().tolist(), targets,
-                                              outputs, sigma=sigma, seed=seed)
+        def forward(fctx, th, call):
+            loss, grad, used = call(th.detach().cpu().tolist())
             fctx.save_for_backward(torch.tensor(grad, dtype=th.dtype, device=th.device))
             fctx.n_used = used
             return th.new_tensor(loss)
@@ -787,7 +786,7 @@ def _ring_chi2_function():
         @staticmethod
         def backward(fctx, gout):
             (grad,) = fctx.saved_tensors
-            return gout * grad, None, None, None, None, None, None
+            return gout * grad, None
 
     return _RingChi2
 
@@ -797,7 +796,9 @@ def ring_chi2(ctx: Context, theta, tracks: DeviceTracks, targets, outputs: Trace
     """Differentiable soft ring chi^2: a torch.autograd.Function over the
     10 parameters (8 tile tilts, radius of curvature, n - 1); its backward
     is the gradient from rich_trace_grad's adjoint pass."""
-    return _ring_chi2_function().apply(theta, ctx, tracks, targets, outputs, sigma, seed)
+    # the other arguments stay outside of apply, so that autograd sees theta alone
+    return _ring_chi2_function().apply(
+        theta, lambda th: ctx.trace_grad(tracks, th, targets, outputs, sigma=sigma, seed=seed))
 
 
 def rich_trace_grad(ctx: Context, tracks, theta, targets, outputs, **kw):
