@@ -103,10 +103,12 @@ struct rich_ctx {
     bool slot_zeroed[2] = {true, true};
     bool capturing = false;                // inside rich_graph_capture
     // kernel timing (rich_set_timing): events around the kernels of the
-    // last rich_emit (0 yield, 1 ordering, 2 end) and rich_trace (3 trace,
-    // 4 refinement, 5 end); recorded[k]: event k belongs to the last call
+    // last rich_emit (0 yield, 1 its end, 2 the ordering's end) and rich_trace
+    // (3 trace, 4 refinement, 5 end). The ordering starts at event tev_order: 1,
+    // or 6 when photon arrays or the host's read of the total come between
     bool timing = false;
-    cudaEvent_t tev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t tev[7] = {};
+    int tev_order = 1;
     bool tev_emit = false, tev_trace = false, tev_refine = false;
     // counting build of the trace (rich_trace_work): 6 device tallies
     unsigned long long *d_work = nullptr;
@@ -1010,6 +1012,7 @@ RICH_API rich_status rich_emit(rich_ctx *ctx, const rich_tracks *t,
                                          /*defer_scan=*/!(n_photons || out));
         if (st != RICH_OK) return st;
     }
+    if (timed) RICH_CUDA(cudaEventRecord(ctx->tev[1], ctx->stream));
     // the arrays are written before the host reads the total, so the GPU does not
     // wait for it (arrays that are missing or too small are refused below,
     // unwritten)
@@ -1025,7 +1028,10 @@ RICH_API rich_status rich_emit(rich_ctx *ctx, const rich_tracks *t,
         ctx->known_total = std::max<uint64_t>(ctx->known_total, *ctx->h_total);
         if (n_photons) *n_photons = *ctx->h_total;
     }
-    if (timed) RICH_CUDA(cudaEventRecord(ctx->tev[1], ctx->stream));
+    if (timed) {
+        ctx->tev_order = n_photons || out ? 6 : 1;
+        if (ctx->tev_order == 6) RICH_CUDA(cudaEventRecord(ctx->tev[6], ctx->stream));
+    }
     {
         const rich_status st = order_photons(ctx);
         if (st != RICH_OK) return st;
@@ -1286,7 +1292,7 @@ RICH_API rich_status rich_kernel_times(rich_ctx *ctx, rich_kernel_ms *out) {
     if (ctx->tev_emit) {
         RICH_CUDA(cudaEventSynchronize(ctx->tev[2]));
         RICH_CUDA(cudaEventElapsedTime(&out->yield, ctx->tev[0], ctx->tev[1]));
-        RICH_CUDA(cudaEventElapsedTime(&out->order, ctx->tev[1], ctx->tev[2]));
+        RICH_CUDA(cudaEventElapsedTime(&out->order, ctx->tev[ctx->tev_order], ctx->tev[2]));
     }
     if (ctx->tev_trace) {
         RICH_CUDA(cudaEventSynchronize(ctx->tev[5]));

@@ -130,3 +130,24 @@ def test_kernel_timing():
     ctx.trace(out, precision=rich.PREC_REFINE64)
     assert ctx.kernel_times() == {"yield": -1.0, "order": -1.0, "trace": -1.0, "refine": -1.0}
     ctx.close()
+
+
+def test_yield_time_is_without_the_photon_arrays():
+    """The yield time is that of the count and scan whether or not the emission
+    writes photon arrays. 40 bytes a photon take more than 80 us here at 8 TB/s, the
+    memory's nominal rate; the bound is half of that above the time without."""
+    scene, ctx, _, _ = _setup(1)
+    dt = rich.DeviceTracks(W.pion_tracks(60_000, seed=3))
+    n = ctx.emit(dt, 0.0014, seed=4, sync=True)
+    assert 40 * n / 8e12 > 80e-6
+    pb = rich.PhotonBuffers(n)
+    ctx.set_timing(True)
+    times = {}
+    for arrays in (None, pb):
+        t = []
+        for _ in range(5):
+            assert ctx.emit(dt, 0.0014, seed=4, photons=arrays, sync=True) == n
+            t.append(ctx.kernel_times()["yield"])
+        times[arrays is None] = min(t)
+    ctx.close()
+    assert times[True] > 0 and times[False] < times[True] + 0.040, times
