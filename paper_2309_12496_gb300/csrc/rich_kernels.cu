@@ -1845,8 +1845,8 @@ __device__ __forceinline__ ff shfl_xor_ff(ff a, int o) {
 }
 
 // Event sums (hits, sum u, sum v, sum lambda) of the lanes of a converged
-// warp: the taking lanes of one (event, plane) key add up pairwise in
-// double-word arithmetic (~1e-14 relative), all keys at once: in every round a
+// warp: the taking lanes of one (event, plane) key add up pairwise in double-word
+// arithmetic (five additions of 3 x 2^-48 at most), all keys at once: in every round a
 // lane takes the sum of its next peer, and every second one of those left has
 // been taken. The key's first lane then adds to the sums with one FP64 atomic
 // per component, so the accumulation over warps is FP64; the hit count is the
@@ -2579,102 +2579,122 @@ k_trace(TraceArgs A) {
 // its instructions are FP32 additions) and by instruction fetch at small counts.
 // With the fused forms and 32 warps per SM instead of 16, 5.0e5 RICH1 hits take 105
 // -> 80 us, 3.2e6 RICH2 hits 570 -> 436 us, 1.2e6 scintillator hits 268 -> 162 us.
-constexpr int kRefineThreads = 256;
+//
+// Event sums: with few keys (one event) each thread sums its own hits per key, and
+// the warp's butterfly (15 double-word additions and shuffles per key) runs once per
+// kOwnChunks chunks instead of once per chunk: 5.0e5 RICH1 hits 80 -> 63 us, 3.2e6
+// RICH2 hits 436 -> 337 us; more than four keys would take shared memory from the
+// block beside this one. A sum passes at most kOwnChunks + 5 double-word additions
+// (3 x 2^-48 each) before it is FP64, whatever the number of hits. In FP64 follow
+// the additions of a block's warps in shared memory and of the blocks in global
+// memory, and the latter make up the error, so two blocks of 512 threads per SM and
+// not four of 256: rms against the exact sum of the hits, in 2^-48 of the sum of their
+// magnitudes, 0.12 and 0.16 (RICH2, 8.9e5 hits), 0.11 and 0.15 (RICH1, 5.0e5 hits),
+// where FP64 additions of every chunk's sum in 304 blocks left 0.12 and 0.11. Refinement
+// of 5.0e6 hits 444 us (four blocks of 256: 460 us), a step of 1000 tracks 80.1 us
+// (79.4 us).
+constexpr int kRefineThreads = 512;
 constexpr int kOwnKeys = 4;
+constexpr int kOwnChunks = 32;
+constexpr size_t kOwnBytes = (3 * sizeof(ff) + sizeof(uint32_t)) * kRefineThreads;   // per key
+__host__ __device__ __forceinline__ bool refine_own(const TraceParams &P, int n_planes) {
+    return P.event_sums && (int64_t)P.n_hist_events * n_planes <= kOwnKeys;
+}
 template <bool EXT>
-__global__ void __launch_bounds__(kRefineThreads, 4)
+__global__ void __launch_bounds__(kRefineThreads, 2)
 k_refine(SceneView sc, EmitView em, ExtView ext, TraceParams P, Counters *ctr) {
     __shared__ double s_es_tab[kSmemKeys * 4];
     double *const s_es = es_table_on(sc, P) ? s_es_tab : nullptr;
     for (int i = threadIdx.x; i < kSmemKeys * 4; i += blockDim.x) s_es_tab[i] = 0.0;
-    // with few keys (one event) each thread sums its own hits, per key, and
-    // the warp's butterfly (15 double-word additions and shuffles per key) runs
-    // once at the end instead of once per chunk: 5.0e5 RICH1 hits 80 -> 63 us,
-    // 3.2e6 RICH2 hits 436 -> 337 us; more than four keys would take shared memory
-    // from the blocks beside this one
-    __shared__ ff s_own[kOwnKeys][3][kRefineThreads];
-    __shared__ uint32_t s_own_n[kOwnKeys][kRefineThreads];
-    const int n_keys = s_es ? (int)P.n_hist_events * sc.n_planes : 0;
-    const bool own = s_es && n_keys <= kOwnKeys;
-    if (own)
-        for (int k = 0; k < n_keys; ++k) {
-            for (int q = 0; q < 3; ++q) s_own[k][q][threadIdx.x] = ffv(0.0f);
-            s_own_n[k][threadIdx.x] = 0u;
-        }
+    const bool own = refine_own(P, sc.n_planes);
+    const int n_keys = own ? (int)P.n_hist_events * sc.n_planes : 0;
+    // dynamic shared memory: [key][u, v, lambda][thread] sums, [key][thread] counts
+    ff(*const s_own)[3][kRefineThreads] = reinterpret_cast<ff(*)[3][kRefineThreads]>(rich_dsmem);
+    uint32_t(*const s_own_n)[kRefineThreads] =
+        reinterpret_cast<uint32_t(*)[kRefineThreads]>(s_own + n_keys);
+    for (int k = 0; k < n_keys; ++k) {
+        for (int q = 0; q < 3; ++q) s_own[k][q][threadIdx.x] = ffv(0.0f);
+        s_own_n[k][threadIdx.x] = 0u;
+    }
     __syncthreads();
     grid_dep_wait();                     // the trace has ended
     const uint64_t n_hits = ctr->hits < P.hit_capacity ? ctr->hits : P.hit_capacity;
     const uint64_t n_chunks = (n_hits + 31) / 32;
     const uint64_t n_warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     const int lane = threadIdx.x & 31;
-    for (uint64_t c = blockIdx.x + (uint64_t)gridDim.x * (threadIdx.x >> 5); c < n_chunks;
-         c += n_warps) {
-        const uint64_t i = c * 32 + (uint64_t)lane;
-        const bool on = i < n_hits;
-        ff uf = ffv(0.0f), vf = ffv(0.0f);
-        int plane = 0;
-        uint32_t event = 0;
-        float lam = 0.0f;
-        if (on) {
-            const rich_hit h = P.hits[i];
-            const RefineRec rr = P.refine[i];
-            ff3 o, d;
-            if (EXT) {
-                const uint32_t g = rr.index;
-                o = ff3v(ext.x[g], ext.y[g], ext.z[g]);
-                d = ff3_normalized(ff3v(ext.dx[g], ext.dy[g], ext.dz[g]));
-            } else {
-                emit_ff(em.tracks[rr.index], em.frame[rr.index], em.cos_sin[rr.index], h.photon,
-                        h.lambda, em, o, d);
+    for (uint64_t c = blockIdx.x + (uint64_t)gridDim.x * (threadIdx.x >> 5); c < n_chunks;) {
+        for (int turn = 0; turn < kOwnChunks && c < n_chunks; ++turn, c += n_warps) {
+            const uint64_t i = c * 32 + (uint64_t)lane;
+            const bool on = i < n_hits;
+            ff uf = ffv(0.0f), vf = ffv(0.0f);
+            int plane = 0;
+            uint32_t event = 0;
+            float lam = 0.0f;
+            if (on) {
+                const rich_hit h = P.hits[i];
+                const RefineRec rr = P.refine[i];
+                ff3 o, d;
+                if (EXT) {
+                    const uint32_t g = rr.index;
+                    o = ff3v(ext.x[g], ext.y[g], ext.z[g]);
+                    d = ff3_normalized(ff3v(ext.dx[g], ext.dy[g], ext.dz[g]));
+                } else {
+                    emit_ff(em.tracks[rr.index], em.frame[rr.index], em.cos_sin[rr.index], h.photon,
+                            h.lambda, em, o, d);
+                }
+                replay_ff(sc, o, d, rr, h.lambda, uf, vf);
+                int ix, iy;
+                pixel_of_ff(sc.rects[rr.det_rect], uf, vf, ix, iy);
+                P.hits[i].u = ff_to_double(uf);
+                P.hits[i].v = ff_to_double(vf);
+                P.hits[i].ix = (uint16_t)ix;
+                P.hits[i].iy = (uint16_t)iy;
+                plane = h.plane;
+                event = h.event;
+                lam = h.lambda;
+                bin_hit(sc, P, event, plane, ix, iy);
             }
-            replay_ff(sc, o, d, rr, h.lambda, uf, vf);
-            int ix, iy;
-            pixel_of_ff(sc.rects[rr.det_rect], uf, vf, ix, iy);
-            P.hits[i].u = ff_to_double(uf);
-            P.hits[i].v = ff_to_double(vf);
-            P.hits[i].ix = (uint16_t)ix;
-            P.hits[i].iy = (uint16_t)iy;
-            plane = h.plane;
-            event = h.event;
-            lam = h.lambda;
-            bin_hit(sc, P, event, plane, ix, iy);
+            if (!own) {
+                add_event_sums_ff(sc, P, on, event, plane, uf, vf, lam, s_es);
+            } else if (on && event < P.n_hist_events) {
+                const int k = (int)event * sc.n_planes + plane;
+                ff(*a)[kRefineThreads] = s_own[k];
+                a[0][threadIdx.x] = ff_add(a[0][threadIdx.x], uf);
+                a[1][threadIdx.x] = ff_add(a[1][threadIdx.x], vf);
+                a[2][threadIdx.x] = ff_add(a[2][threadIdx.x], lam);
+                s_own_n[k][threadIdx.x] += 1u;
+            }
         }
-        if (!own) {
-            add_event_sums_ff(sc, P, on, event, plane, uf, vf, lam, s_es);
-        } else if (on && event < P.n_hist_events) {
-            const int k = (int)event * sc.n_planes + plane;
-            ff(*a)[kRefineThreads] = s_own[k];
-            a[0][threadIdx.x] = ff_add(a[0][threadIdx.x], uf);
-            a[1][threadIdx.x] = ff_add(a[1][threadIdx.x], vf);
-            a[2][threadIdx.x] = ff_add(a[2][threadIdx.x], lam);
-            s_own_n[k][threadIdx.x] += 1u;
-        }
-    }
-    if (own) {
-        // lane 4 k + q keeps sum q of key k, so that the FP64 conversions and the
-        // atomics of all keys are one instruction each (one lane's chain of them
-        // before: 1000 RICH1 tracks 18.4 -> 16.4 us, the call 88.2 -> 86.3 us)
-        ff mine = ffv(0.0f);
-        uint32_t got = 0u;
-        for (int k = 0; k < n_keys; ++k) {
-            const uint32_t n = __reduce_add_sync(kFull, s_own_n[k][threadIdx.x]);
-            if (n == 0) continue;        // uniform in the warp
-            ff a[3];
+        if (own) {
+            // lane 4 k + q keeps sum q of key k, so that the FP64 conversions and the
+            // atomics of all keys are one instruction each (one lane's chain of them
+            // before: 1000 RICH1 tracks 18.4 -> 16.4 us, the call 88.2 -> 86.3 us)
+            ff mine = ffv(0.0f);
+            uint32_t got = 0u;
+            for (int k = 0; k < n_keys; ++k) {
+                const uint32_t n = __reduce_add_sync(kFull, s_own_n[k][threadIdx.x]);
+                if (n == 0) continue;        // uniform in the warp
+                ff a[3];
 #pragma unroll
-            for (int q = 0; q < 3; ++q) a[q] = s_own[k][q][threadIdx.x];
+                for (int q = 0; q < 3; ++q) {
+                    a[q] = s_own[k][q][threadIdx.x];
+                    s_own[k][q][threadIdx.x] = ffv(0.0f);
+                }
+                s_own_n[k][threadIdx.x] = 0u;
 #pragma unroll 1
-            for (int o = 16; o > 0; o >>= 1)
+                for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-                for (int q = 0; q < 3; ++q) a[q] = ff_add(a[q], shfl_xor_ff(a[q], o));
-            if ((lane >> 2) == k) {
-                got = n;
+                    for (int q = 0; q < 3; ++q) a[q] = ff_add(a[q], shfl_xor_ff(a[q], o));
+                if ((lane >> 2) == k) {
+                    got = n;
 #pragma unroll
-                for (int q = 0; q < 3; ++q)
-                    if ((lane & 3) == q + 1) mine = a[q];
+                    for (int q = 0; q < 3; ++q)
+                        if ((lane & 3) == q + 1) mine = a[q];
+                }
             }
+            if (got != 0u)
+                atomicAdd(s_es + lane, (lane & 3) == 0 ? (double)got : ff_to_double(mine));
         }
-        if (got != 0u)
-            atomicAdd(s_es + lane, (lane & 3) == 0 ? (double)got : ff_to_double(mine));
     }
     __syncthreads();
     if (s_es) es_table_flush(sc, P, s_es);
@@ -2684,15 +2704,22 @@ cudaError_t launch_refine(const SceneView &sc, const EmitView *em, const ExtView
                           const TraceParams &p, Counters *counters, int n_sm,
                           cudaStream_t s) {
     if (p.hit_capacity == 0) return cudaSuccess;
-    // every block resident at once (four 256-thread blocks per SM)
+    // every block resident at once (two 512-thread blocks per SM)
     uint64_t blocks = (p.hit_capacity + kRefineThreads - 1) / kRefineThreads;
-    const uint64_t cap = (uint64_t)n_sm * 4;
+    const uint64_t cap = (uint64_t)n_sm * 2;
     if (blocks > cap) blocks = cap;
+    const size_t smem =
+        refine_own(p, sc.n_planes) ? kOwnBytes * (size_t)p.n_hist_events * sc.n_planes : 0;
+    const void *const f = ext ? (const void *)k_refine<true> : (const void *)k_refine<false>;
+    if (smem > 44 * 1024) {              // beside 2 KB of static shared memory
+        const cudaError_t e = ensure_dyn_smem(f, smem);
+        if (e != cudaSuccess) return e;
+    }
     if (ext)
-        return launch_pdl(k_refine<true>, (unsigned)blocks, kRefineThreads, 0, s, sc,
+        return launch_pdl(k_refine<true>, (unsigned)blocks, kRefineThreads, smem, s, sc,
                           em ? *em : EmitView{}, *ext, p, counters);
-    return launch_pdl(k_refine<false>, (unsigned)blocks, kRefineThreads, 0, s, sc, *em, ExtView{}, p,
-                      counters);
+    return launch_pdl(k_refine<false>, (unsigned)blocks, kRefineThreads, smem, s, sc, *em, ExtView{},
+                      p, counters);
 }
 
 // ============================================================== adjoint
