@@ -548,6 +548,45 @@ int staged_nodes(const rich_ctx *ctx, int opt, int threads, bool proxies) {
     return std::min(n, (int)ctx->sc.n_nodes);
 }
 
+// Blocks per SM that a trace kernel reaches (queried once), 0 if none.
+int trace_occupancy(rich_ctx *ctx, bool ext, bool refine, bool proxy, int cls, int threads,
+                    size_t smem) {
+    if (smem > (size_t)ctx->smem_optin) return 0;
+    const auto key = std::make_tuple(ext, refine, proxy, cls, threads, smem);
+    auto it = ctx->occupancy.find(key);
+    if (it == ctx->occupancy.end())
+        it = ctx->occupancy
+                 .emplace(key, trace_blocks_per_sm(ext, refine, cls, threads, smem, proxy)).first;
+    return it->second;
+}
+
+// Launch shape of a trace on scene sc: threads, build, staged nodes and shared
+// memory, and the blocks per SM (0: it does not fit). Nodes asked for that fit beside
+// the state of 512 threads and not of 1024 (1364 to 1575 on RICH1) are staged by blocks
+// of 512, unless the threads are asked for too. The proxies and the groups' bounding
+// spheres have taken a share of the shared memory (1.3 KB at most): nodes that fit
+// without it are reduced by it.
+int fit_trace(rich_ctx *ctx, const SceneView &sc, const rich_trace_opts &o, bool ext, bool refine,
+              bool proxy, LaunchShape &shape, int &nodes) {
+    const size_t share = sizeof(DevProxy) * sc.n_proxies + 4 * sizeof(float) * sc.n_groups;
+    for (int threads = o.block_threads ? o.block_threads : kDefaultThreads;; threads = 512) {
+        shape.threads = threads;
+        shape.cls = trace_shape_class(threads, o.wide_regs != 0);
+        nodes = staged_nodes(ctx, o.bvh_smem_nodes, threads, proxy);
+        auto fits = [&](size_t smem) {
+            return trace_occupancy(ctx, ext, refine, proxy, shape.cls, threads, smem);
+        };
+        shape.smem = trace_smem_bytes(sc, nodes, threads, shape.cls);
+        int bps = fits(shape.smem);
+        if (bps < 1 && nodes > 0 && fits(shape.smem - share) > 0) {
+            nodes = std::max(0, nodes - (int)((share + sizeof(DevNode) - 1) / sizeof(DevNode)));
+            shape.smem = trace_smem_bytes(sc, nodes, threads, shape.cls);
+            bps = fits(shape.smem);
+        }
+        if (bps > 0 || o.block_threads || threads == 512) return bps;
+    }
+}
+
 // A scene of rectangles alone: a photon's step costs the same wherever it goes,
 // so a warp refills when half its lanes are idle (photons make 1 to 8 bounces in
 // a mirror box): scintillator box, 4e6 photons, chunks of 32, 792 -> 587 us (with
@@ -1121,8 +1160,6 @@ static rich_status trace_impl(rich_ctx *ctx, const rich_photons *in, const rich_
          ctx->table_kind[ctx->spectrum] != RICH_TABLE_CDF))
         return fail(ctx, RICH_ERR_STATE,
                     "rich_trace: the emission's spectrum table is not in the current scene");
-    const int cls = trace_shape_class(threads, o->wide_regs != 0);
-    const int smem_nodes = staged_nodes(ctx, o->bvh_smem_nodes, threads, ctx->sc.n_proxies > 0 && !work);
     DeviceGuard guard(ctx->device);
     const bool refine = o->precision == RICH_PREC_REFINE64;
     const uint64_t hit_cap = out->hits ? out->hit_capacity : 0;
@@ -1166,31 +1203,21 @@ static rich_status trace_impl(rich_ctx *ctx, const rich_photons *in, const rich_
     p.fate = out->fate;
     p.fate_capacity = out->fate ? out->fate_capacity : 0;
     p.refine = ctx->d_refine;
-    p.smem_nodes = smem_nodes;
     p.wait_limit = trace_wait_limit(o->wait_limit);
     p.n_prefilter = o->n_prefilter;
     for (int k = 0; k < 4; ++k) p.prefilter_tables[k] = k < o->n_prefilter ? o->prefilter_tables[k] : 0;
     LaunchShape shape;
-    shape.threads = threads;
-    shape.smem = trace_smem_bytes(ctx->sc, smem_nodes, threads, cls);
-    shape.cls = cls;
-    if (shape.smem > (size_t)ctx->smem_optin)
-        return fail(ctx, RICH_ERR_ARG, "rich_trace: staged BVH nodes exceed shared memory");
-    int bps = o->blocks_per_sm;
-    {
-        const bool proxy = ctx->sc.n_proxies > 0 && !work;
-        const auto key = std::make_tuple(in != nullptr, refine, proxy, cls, threads, shape.smem);
-        auto it = ctx->occupancy.find(key);
-        if (it == ctx->occupancy.end())
-            it = ctx->occupancy.emplace(key, trace_blocks_per_sm(in != nullptr, refine, cls,
-                                                                 threads, shape.smem, proxy)).first;
-        if (it->second < 1)
-            return fail(ctx, RICH_ERR_ARG, "rich_trace: launch shape does not fit on an SM");
-        if (!bps || bps > it->second) bps = it->second;
-    }
+    int bps = fit_trace(ctx, ctx->sc, *o, in != nullptr, refine, ctx->sc.n_proxies > 0 && !work, shape,
+                        p.smem_nodes);
+    if (bps < 1)
+        return fail(ctx, RICH_ERR_ARG,
+                    shape.smem > (size_t)ctx->smem_optin
+                        ? "rich_trace: staged BVH nodes exceed shared memory"
+                        : "rich_trace: launch shape does not fit on an SM");
+    if (o->blocks_per_sm && o->blocks_per_sm < bps) bps = o->blocks_per_sm;
     shape.blocks = std::max(1, bps) * ctx->n_sm;
     if (work) {
-        if (in || !refine || !trace_count_shape_ok(cls))
+        if (in || !refine || !trace_count_shape_ok(shape.cls))
             return fail(ctx, RICH_ERR_ARG,
                         "rich_trace_work: counts the fused-emission trace with refinement in "
                         "the wide (up to 896 threads) or the 1024-thread shape");
@@ -1426,8 +1453,6 @@ RICH_API rich_status rich_trace_grad(rich_ctx *ctx, const rich_tracks *t,
         RICH_CUDA(cudaMallocHost(&ctx->h_acc, sizeof(double) * 12));
     }
     const int threads = fo.block_threads ? fo.block_threads : kDefaultThreads;
-    const int cls = trace_shape_class(threads, fo.wide_regs != 0);
-    const int smem_nodes = staged_nodes(ctx, fo.bvh_smem_nodes, threads, sv.n_proxies > 0);
     TraceParams p{};
     p.precision = RICH_PREC_REFINE64;
     p.max_bounces = fo.max_bounces;
@@ -1443,17 +1468,12 @@ RICH_API rich_status rich_trace_grad(rich_ctx *ctx, const rich_tracks *t,
     p.fate = out->fate;
     p.fate_capacity = out->fate ? out->fate_capacity : 0;
     p.refine = ctx->d_refine;
-    p.smem_nodes = smem_nodes;
     p.wait_limit = trace_wait_limit(fo.wait_limit);
     if (p.max_bounces < 1 || p.max_bounces > RICH_MAX_BOUNCES || p.max_steps < 1 ||
         p.max_steps > RICH_MAX_STEPS || threads % 32 || threads > 1024)
         return fail(ctx, RICH_ERR_ARG, "rich_trace_grad: trace options out of range");
     LaunchShape shape;
-    shape.threads = threads;
-    shape.cls = cls;
-    shape.smem = trace_smem_bytes(sv, smem_nodes, threads, cls);
-    const int bps = trace_blocks_per_sm(false, true, cls, threads, shape.smem,
-                                        sv.n_proxies > 0);
+    const int bps = fit_trace(ctx, sv, fo, false, true, sv.n_proxies > 0, shape, p.smem_nodes);
     if (bps < 1) return fail(ctx, RICH_ERR_ARG, "rich_trace_grad: launch shape does not fit");
     shape.blocks = bps * ctx->n_sm;
     Counters *ctr = nullptr, *ctr_next = nullptr;

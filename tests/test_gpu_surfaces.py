@@ -80,3 +80,66 @@ def test_rays_from_everywhere_match_the_oracle(name, reach):
     stats = P.compare(gpu, ref, None, P.TOL_UV_REFINE, name=f"everywhere_{name}_{reach}",
                       keys=(arrays["event"], arrays["track"], arrays["photon"]))
     assert stats["hits"] > 0
+
+
+# the most staged nodes of RICH1 that fit in 227 KB beside 1024, 512 and 896 threads'
+# state and the small tables, without the surface proxies' 512 bytes
+@pytest.mark.parametrize("knobs,most", [
+    ({}, 1575), (dict(block_threads=512), 1575), (dict(block_threads=1024), 1367),
+    (dict(block_threads=896, wide_regs=1), 1419), (dict(block_threads=256), 1783)])
+@pytest.mark.parametrize("precision", [rich.PREC_REFINE64, rich.PREC_FP32])
+def test_staged_nodes_up_to_the_shared_memory(knobs, most, precision):
+    """A number of staged nodes is taken up to what the shared memory holds and
+    refused above it, and does not change what is traced."""
+    scene = W.rich1_scene(meshed=True)
+    ctx = rich.Context(0)
+    ctx.init_geometry(scene)
+    dt = rich.DeviceTracks(W.pion_tracks(30, seed=3))
+    n = ctx.emit(dt, 0.0014, seed=4)
+    out = rich.TraceOutputs(n, scene.pixels_per_event, len(scene.planes), 1, n)
+    got = []
+    for nodes in (-1, 1300, most - 4, most):
+        ctx.emit(dt, 0.0014, seed=4)
+        out.clear()
+        ctx.trace(out, precision=precision, bvh_smem_nodes=nodes, **knobs)
+        n_hits, _ = ctx.hits()
+        got.append((np.sort(out.hits_numpy(n_hits), order=["event", "track", "photon"]),
+                    out.fate.cpu().numpy().copy()))
+    with pytest.raises(rich.RichError):
+        ctx.trace(out, precision=precision, bvh_smem_nodes=most + 1, **knobs)
+    ctx.close()
+    assert len(got[0][0]) > 1000
+    for hits, fate in got[1:]:
+        np.testing.assert_array_equal(hits, got[0][0])
+        np.testing.assert_array_equal(fate, got[0][1])
+
+
+def test_staged_nodes_of_a_gradient():
+    """The same limits hold for the gradient's forward pass."""
+    scene = W.rich1_scene(meshed=True)
+    ctx = rich.Context(0)
+    ctx.init_geometry(scene)
+    tracks = W.pion_tracks(30, seed=3)
+    dt = rich.DeviceTracks(tracks)
+    n = ctx.emit(dt, 0.0014, seed=4)
+    planes = len(scene.planes)
+    out = rich.TraceOutputs(n, scene.pixels_per_event, planes, 1, n)
+    ctx.trace(out)
+    n_hits, _ = ctx.hits()
+    h = out.hits_numpy(n_hits)
+    tg = torch.from_numpy(W.ring_targets(30, planes, h["track"].astype(np.int64), h["plane"],
+                                         h["u"] + 1.0, h["v"])).cuda()
+    th = W.nominal_theta(scene, 0.0014)
+    th[8] = 2000.0                       # (no tiles to apply it to)
+    res = {}
+    for nodes in (-1, 1571, 1575):
+        res[nodes] = ctx.trace_grad(dt, th, tg, out, seed=4, bvh_smem_nodes=nodes)
+    with pytest.raises(rich.RichError):
+        ctx.trace_grad(dt, th, tg, out, seed=4, bvh_smem_nodes=1576)
+    ctx.close()
+    loss, grad, used = res[-1]
+    assert used > 500
+    for nodes in (1571, 1575):
+        # sums of up to 1e5 FP64 terms in another order
+        assert res[nodes][0] == pytest.approx(loss, rel=1e-10) and res[nodes][2] == used
+        np.testing.assert_allclose(res[nodes][1], grad, rtol=1e-8, atol=1e-8 * np.abs(grad).max())
