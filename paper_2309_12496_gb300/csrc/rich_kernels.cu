@@ -1506,10 +1506,10 @@ __device__ __noinline__ void nearest_bvh_far(const SceneView &sc, const DevNode 
 // trace of RICH1, 10^4 tracks, 1058 -> 725 us, of RICH2, 1.2 x 10^5 tracks,
 // 9.15 -> 6.01 ms, 10^6 caller photons on RICH1 463 -> 296 us a call.
 // A proxy whose mesh the ray passes by is left by one test of the sphere that
-// bounds it (RICH1, 10^4 tracks, 518 -> 485 us; RICH2 3.99 -> 3.78 ms). Up to two
-// crossings with cells are kept, nearest first (a third leaves the ray
-// to the BVH unless a nearer hit settles it), and their triangles are tested
-// after the last proxy, so that lanes whose mirrors differ test theirs together.
+// bounds it (RICH1, 10^4 tracks, 518 -> 485 us; RICH2 3.99 -> 3.78 ms). The triangles
+// of the cells that proxy_cells keeps are tested after the last proxy, so that
+// lanes whose mirrors differ test theirs together; a third crossing leaves the
+// ray to the BVH unless a nearer hit settles it.
 template <bool EXT>
 __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemScene &S, f3 o, f3 d,
                                                 int skip, int skip_ref, uint32_t skip_px,
@@ -1518,58 +1518,10 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
     // unit vectors, are outside the proxies' bounds
     if (!(dot3(o, o) <= sc.proxy_o2_max)) return false;
     if (EXT && !(fabsf(dot3(d, d) - 1.0f) <= 2.0e-6f)) return false;
-    const float kInf = __int_as_float(0x7f800000);
-    float t0 = kInf, t1 = kInf, t2 = kInf;      // nearest three
-    int c0 = -1, c1 = -1;
-    auto keep = [&](float t, int c) {
-        t = c >= 0 ? t : kInf;
-        const bool l0 = t < t0, l1 = t < t1;
-        t2 = fminf(t2, l1 ? t1 : t);
-        c1 = l0 ? c0 : (l1 ? c : c1);
-        t1 = l0 ? t0 : (l1 ? t : t1);
-        c0 = l0 ? c : c0;
-        t0 = l0 ? t : t0;
-    };
-    unsigned entering = 0;
-    bool all = true;
-    // the proxy of the surface just left: passed over when that is its only
-    // surface; when its surfaces lie apart, its entry crossing (the start)
-    // lists none but the one left (RICH1, 10^4 tracks, 482 -> 457 us; RICH2 3.76
-    // -> 3.54 ms)
-    const int left = (int)(skip_px & kProxyIndex) - 1;
-    const int own = skip_px & kProxySingle ? left : -1;
-    const unsigned no_entry = skip_px & kProxyApart ? 1u << left : 0u;
-#pragma unroll 1
-    for (int i = 0; i < S.n_proxies; ++i) {
-        const DevProxy &P = S.proxies()[i];
-        if (proxy_misses(P, o.x, o.y, o.z, d.x, d.y, d.z, b.t) | (i == own)) continue;
-        float t;
-        bool sure;
-        int c;
-        if (i < sc.n_proxy_planes) {
-            c = proxy_plane(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure);
-        } else {
-            float sb, h2;
-            bool ent;
-            c = proxy_sphere(P, o.x, o.y, o.z, d.x, d.y, d.z, t_min, b.t, t, sure, ent, sb, h2);
-            entering |= (unsigned)ent << i;
-        }
-        all = all & sure;
-        keep(t, c);
-    }
-    entering &= ~no_entry;
-    while (entering) {
-        const DevProxy &P = S.proxies()[__ffs(entering) - 1];
-        entering &= entering - 1u;
-        const float wx = o.x - P.cx, wy = o.y - P.cy, wz = o.z - P.cz;
-        const float sb = fmaf(wx, d.x, fmaf(wy, d.y, wz * d.z));
-        const float qx = fmaf(-sb, d.x, wx), qy = fmaf(-sb, d.y, wy), qz = fmaf(-sb, d.z, wz);
-        const float h2 = P.r2 - fmaf(qx, qx, fmaf(qy, qy, qz * qz));
-        float t;
-        const int c = proxy_sphere_side(P, wx, wy, wz, d.x, d.y, d.z, sb, h2, -1.0f, t_min, b.t, t,
-                                        true);
-        keep(t, c);
-    }
+    const ProxyCells q = proxy_cells(S, sc.n_proxy_planes, o.x, o.y, o.z, d.x, d.y, d.z, skip_px,
+                                     t_min, b.t);
+    bool all = q.sure;
+    int c0 = q.c0;
     if (c0 >= 0) {
         const Ray r = make_ray(o, d);
 #pragma unroll 1
@@ -1578,16 +1530,16 @@ __device__ __forceinline__ bool nearest_proxies(const SceneView &sc, const SmemS
             const bool list = c.y < -1;
             const int n = list ? (c.y & 0x7FFFFFFF) : (c.x >= 0) + (c.y >= 0);
 #pragma unroll 1
-            for (int q = 0; q < n; ++q) {
-                const int tri = list ? __ldg(sc.proxy_lists + c.x + q) : (q ? c.y : c.x);
+            for (int m = 0; m < n; ++m) {
+                const int tri = list ? __ldg(sc.proxy_lists + c.x + m) : (m ? c.y : c.x);
                 const Tri T = load_tri(sc.tris + tri);
                 if (T.prim == skip || T.pad == skip_ref) continue;
                 test_tri(sc, r, T, tri, t_min, b);
             }
-            if (c1 < 0 || t1 > b.t + sc.proxy_dt) break;
-            c0 = c1;
+            if (q.c1 < 0 || q.t1 > b.t + sc.proxy_dt) break;
+            c0 = q.c1;
         }
-        all = all && t2 > b.t + sc.proxy_dt;
+        all = all && q.t2 > b.t + sc.proxy_dt;
     }
     return all;
 }

@@ -120,6 +120,75 @@ RICH_HD int proxy_sphere(const DevProxy &P, float ox, float oy, float oz, float 
     return proxy_sphere_side(P, wx, wy, wz, dx, dy, dz, b, h2, 1.0f, t_min, t_max, t, meets);
 }
 
+// The cells that a ray has to look up: of its two nearest crossings that have one
+// (c0, c1, at t0 <= t1; -1: none), and the distance of a third (infinity: none).
+struct ProxyCells {
+    int c0, c1;
+    float t0, t1, t2;
+    bool sure;             // the margins hold for the ray at every proxy
+};
+
+// S: n_proxies and proxies(), the planes first. skip_px: the proxy code of the
+// triangle just left, or 0. Its proxy is passed over when that is its only surface;
+// when its surfaces lie apart, its entry crossing (the start) lists none but the
+// one left (RICH1, 10^4 tracks, 482 -> 457 us; RICH2 3.76 -> 3.54 ms).
+template <class Proxies>
+RICH_HD ProxyCells proxy_cells(const Proxies &S, int n_planes, float ox, float oy, float oz,
+                               float dx, float dy, float dz, uint32_t skip_px, float t_min,
+                               float t_max) {
+    const float kInf = HUGE_VALF;
+    ProxyCells r{-1, -1, kInf, kInf, kInf, true};
+    auto keep = [&](float t, int c) {
+        t = c >= 0 ? t : kInf;
+        const bool l0 = t < r.t0, l1 = t < r.t1;
+        r.t2 = fminf(r.t2, l1 ? r.t1 : t);
+        r.c1 = l0 ? r.c0 : (l1 ? c : r.c1);
+        r.t1 = l0 ? r.t0 : (l1 ? t : r.t1);
+        r.c0 = l0 ? c : r.c0;
+        r.t0 = l0 ? t : r.t0;
+    };
+    unsigned entering = 0;
+    const int left = (int)(skip_px & kProxyIndex) - 1;
+    const int own = skip_px & kProxySingle ? left : -1;
+    const unsigned no_entry = skip_px & kProxyApart ? 1u << left : 0u;
+#pragma unroll 1
+    for (int i = 0; i < S.n_proxies; ++i) {
+        const DevProxy &P = S.proxies()[i];
+        if (proxy_misses(P, ox, oy, oz, dx, dy, dz, t_max) | (i == own)) continue;
+        float t;
+        bool sure;
+        int c;
+        if (i < n_planes) {
+            c = proxy_plane(P, ox, oy, oz, dx, dy, dz, t_min, t_max, t, sure);
+        } else {
+            float sb, h2;
+            bool ent;
+            c = proxy_sphere(P, ox, oy, oz, dx, dy, dz, t_min, t_max, t, sure, ent, sb, h2);
+            entering |= (unsigned)ent << i;
+        }
+        r.sure = r.sure & sure;
+        keep(t, c);
+    }
+    entering &= ~no_entry;
+    while (entering) {
+#ifdef __CUDA_ARCH__
+        const DevProxy &P = S.proxies()[__ffs(entering) - 1];
+#else
+        const DevProxy &P = S.proxies()[__builtin_ctz(entering)];
+#endif
+        entering &= entering - 1u;
+        const float wx = ox - P.cx, wy = oy - P.cy, wz = oz - P.cz;
+        const float sb = fmaf(wx, dx, fmaf(wy, dy, wz * dz));
+        const float qx = fmaf(-sb, dx, wx), qy = fmaf(-sb, dy, wy), qz = fmaf(-sb, dz, wz);
+        const float h2 = P.r2 - fmaf(qx, qx, fmaf(qy, qy, qz * qz));
+        float t;
+        const int c = proxy_sphere_side(P, wx, wy, wz, dx, dy, dz, sb, h2, -1.0f, t_min, t_max, t,
+                                        true);
+        keep(t, c);
+    }
+    return r;
+}
+
 // Host builder. On return `proxies` is empty when some triangle fits no
 // proxy (the scene then uses the BVH alone).
 struct ProxyResult {

@@ -4,7 +4,8 @@ compiled for the host beside the builder.
 The property the trace relies on: a ray that meets a triangle is either left
 to the BVH or finds that triangle in the cell of one of its crossings. Rays
 are aimed at points of every kind of triangle, edges and corners included,
-with FP32 origins and directions; grazing and distant ones too."""
+with FP32 origins and directions; grazing and distant ones too. Rays that have
+just left a facet pass over its surface and still find the next one."""
 import ctypes as C
 import os
 import shutil
@@ -82,16 +83,77 @@ extern "C" int proxy_find(int64_t nt, const float *v, const int32_t *surf, doubl
     *listed = nr ? tests / (double)nr : 0.0;
     return (int)R.proxies.size();
 }
-// The nearest triangle ahead of each ray in FP64, or -1: none, or met within 1e-3
-// of an edge (where FP32 may see its neighbour).
-extern "C" void nearest_tri(int64_t nt, const float *v, int64_t nr, const float *o, const float *d,
-                            int32_t *target, double *t_hit) {
+struct HostProxies {
+    const std::vector<DevProxy> *v;
+    int n_proxies;
+    const DevProxy *proxies() const { return v->data(); }
+};
+// The cells that the trace looks up for rays that have just left triangle
+// from[i]: out 1 when target[i], met at t_hit[i], is listed there (or -1, none), 2 when
+// the ray goes to the BVH. used: proxy codes of the triangles, and the number of rays
+// for which the code passed over a crossing.
+extern "C" int proxy_leave(int64_t nt, const float *v, const int32_t *surf, double extent, int64_t nr,
+                           const float *o, const float *d, const int32_t *from,
+                           const int32_t *target, const double *t_hit, uint8_t *out,
+                           uint32_t *codes, int64_t *used) {
+    BvhResult b;
+    std::string err;
+    if (!build_bvh(v, surf, nt, b, err)) return -1;
+    std::vector<DevTri> T((size_t)nt);
+    std::vector<int> pos((size_t)nt);
+    for (int64_t k = 0; k < nt; ++k) {
+        const int s = b.leaf_order[(size_t)k];
+        std::memset(&T[(size_t)k], 0, sizeof(DevTri));
+        std::memcpy(&T[(size_t)k], v + 9 * (int64_t)s, 36);
+        T[(size_t)k].pad = b.surface_ref[(size_t)k];
+        pos[(size_t)s] = (int)k;
+    }
+    ProxyResult R;
+    build_proxies(T, extent, R);
+    if (R.proxies.empty()) return 0;
+    std::vector<DevProxyCell> cells;
+    for (auto &grid : R.cells) cells.insert(cells.end(), grid.begin(), grid.end());
+    for (int64_t k = 0; k < nt; ++k) codes[k] = R.tri_code[(size_t)pos[(size_t)k]];
+    const HostProxies S{&R.proxies, (int)R.proxies.size()};
+    auto lists = [&](int c, int tri) {
+        if (c < 0) return false;
+        const DevProxyCell &L = cells[(size_t)c];
+        if (L.b >= -1) return L.a == tri || L.b == tri;
+        for (int q = 0; q < (L.b & 0x7FFFFFFF); ++q)
+            if (R.lists[(size_t)L.a + q] == tri) return true;
+        return false;
+    };
+    *used = 0;
+    for (int64_t i = 0; i < nr; ++i) {
+        const float *O = o + 3 * i, *D = d + 3 * i;
+        const uint32_t code = codes[from[i]];
+        const ProxyCells q = proxy_cells(S, R.n_planes, O[0], O[1], O[2], D[0], D[1], D[2], code,
+                                         1e-3f, 3e38f);
+        const ProxyCells q0 = proxy_cells(S, R.n_planes, O[0], O[1], O[2], D[0], D[1], D[2], 0u,
+                                          1e-3f, 3e38f);
+        *used += q.c0 != q0.c0 || q.c1 != q0.c1 || q.t2 != q0.t2 || q.sure != q0.sure;
+        const double t = target[i] < 0 ? 3e38 : t_hit[i];
+        const bool second = q.c1 >= 0 && q.t1 <= t + R.dt_max;
+        out[i] = 0;
+        if (!q.sure || (q.c0 >= 0 && !(q.t2 > t + R.dt_max))) out[i] |= 2;
+        const int tri = target[i] < 0 ? -1 : pos[(size_t)target[i]];
+        if (tri < 0 || lists(q.c0, tri) || (second && lists(q.c1, tri))) out[i] |= 1;
+    }
+    return S.n_proxies;
+}
+// The nearest triangle ahead of each ray in FP64 that is not of the surface of
+// triangle from[i] (from may be null); -1: none; -2: met within 1e-3 of an edge (where
+// FP32 may see its neighbour).
+extern "C" void nearest_tri(int64_t nt, const float *v, const int32_t *surf, int64_t nr,
+                            const float *o, const float *d, const int32_t *from, int32_t *target,
+                            double *t_hit) {
     for (int64_t i = 0; i < nr; ++i) {
         const double O[3] = {o[3 * i], o[3 * i + 1], o[3 * i + 2]};
         const double D[3] = {d[3 * i], d[3 * i + 1], d[3 * i + 2]};
         double best = 1e300;
         target[i] = -1;
         for (int64_t k = 0; k < nt; ++k) {
+            if (from && (k == from[i] || (surf && surf[k] == surf[from[i]]))) continue;
             double a[3], e1[3], e2[3];
             for (int c = 0; c < 3; ++c) {
                 a[c] = O[c] - v[9 * k + c];
@@ -111,7 +173,7 @@ extern "C" void nearest_tri(int64_t nt, const float *v, int64_t nr, const float 
             if (in < -1e-3 || t < 1e-2 || t >= best) continue;
             best = t;
             t_hit[i] = t;
-            target[i] = in >= 1e-3 ? (int32_t)k : -1;
+            target[i] = in >= 1e-3 ? (int32_t)k : -2;
         }
     }
 }
@@ -254,8 +316,9 @@ def test_coarse_facets_are_found_at_the_steepest_crossings(lib, name):
     o = (p - d * rng.uniform(0.2, 1.0, (n, 1)) * radius).astype(np.float32)
     k = np.zeros(n, np.int32)
     t_hit = np.zeros(n)
-    lib.nearest_tri(C.c_int64(len(v)), v.ctypes.data_as(C.c_void_p), C.c_int64(n),
-                    *(a.ctypes.data_as(C.c_void_p) for a in (o, d, k, t_hit)))
+    lib.nearest_tri(C.c_int64(len(v)), v.ctypes.data_as(C.c_void_p), None, C.c_int64(n),
+                    *(a.ctypes.data_as(C.c_void_p) for a in (o, d)), None,
+                    *(a.ctypes.data_as(C.c_void_p) for a in (k, t_hit)))
     on = k >= 0
     assert on.mean() > 0.3
     n_proxies, out, reach = _find(lib, v, surf, float(np.abs(v).max()) + radius, o[on], d[on],
@@ -264,6 +327,89 @@ def test_coarse_facets_are_found_at_the_steepest_crossings(lib, name):
     if n_proxies:
         assert np.all(out != 0), (int((out == 0).sum()), len(out))
         assert 0.1 < reach <= 1.0
+
+
+def _tiles(radius, half, cells, gap):
+    """A square patch of a sphere (or a plane, radius 0) cut into 2 x 2 surfaces, `gap`
+    apart, and a plane of one surface across the light that they send back."""
+    tris, surf = [], []
+    for i, x in enumerate((-1, 1)):
+        for j, y in enumerate((-1, 1)):
+            xs, ys = sorted((x * gap / 2, x * half)), sorted((y * gap / 2, y * half))
+            if radius:
+                t, _ = W._mesh_rect_tile(np.zeros(3), radius, *np.eye(3)[[2, 0, 1]], *xs, *ys,
+                                         cells, cells)
+            else:
+                t = W._mesh_rectangle(np.array([xs[0], ys[0], 300.0]), *np.eye(3)[:2],
+                                      xs[1] - xs[0], ys[1] - ys[0], cells, cells)
+            tris.append(t)
+            surf.append(np.full(len(t), 2 * i + j))
+    t = W._mesh_rectangle(np.array([-half, -1.5 * half, -100.0]), *np.eye(3)[:2], 2.5 * half,
+                          3 * half, 4, 4)
+    return (np.concatenate(tris + [t]).astype(np.float32),
+            np.concatenate(surf + [np.full(len(t), 4)]).astype(np.int32))
+
+
+def _stack():
+    """Five parallel planes with half of their triangles missing, so that a ray looks up
+    cells whose triangles it misses."""
+    t = [W._mesh_rectangle(np.array([0.0, 0.0, 15.0 * k]), *np.eye(3)[:2], 300.0, 300.0, 20, 20)
+         for k in range(5)]
+    t = [x[np.random.default_rng(k).random(len(x)) < 0.5] for k, x in enumerate(t)]
+    return (np.concatenate(t).astype(np.float32),
+            np.repeat(np.arange(5, dtype=np.int32), [len(x) for x in t]))
+
+
+def _meshes(scene):
+    return scene.tri_vertices, scene.tri_surface
+
+
+SINGLE, APART = 0x10, 0x20
+# surfaces, and the codes of their triangles
+LEAVE = {
+    "tiles_apart": (lambda: _tiles(500.0, 200.0, 5, 30.0), {SINGLE, APART}),
+    "tiles_apart_coarse": (lambda: _tiles(500.0, 150.0, 2, 60.0), {SINGLE, APART}),
+    "tiles_touching": (lambda: _tiles(500.0, 200.0, 5, 0.0), {SINGLE, 0}),
+    "flats_apart": (lambda: _tiles(0.0, 200.0, 5, 30.0), {SINGLE, APART}),
+    "flats_touching": (lambda: _tiles(0.0, 200.0, 5, 0.0), {SINGLE, 0}),
+    "stack": (_stack, {SINGLE}),
+    "rich1": (lambda: _meshes(W.rich1_scene(tiles_per_edge=8, flat_cells=(8, 6))), {SINGLE, APART}),
+    "rich2": (lambda: _meshes(W.rich2_scene(hex_subdiv=6)), {SINGLE, 0}),
+}
+
+
+@pytest.mark.parametrize("name", sorted(LEAVE))
+def test_a_ray_that_leaves_a_facet_finds_the_next_surface(lib, name):
+    """Rays that start on a facet, in every direction (half of them at other
+    triangles): the surface just left is passed over with its proxy or with the
+    entry crossing, and the nearest triangle of any other surface is still found."""
+    make, codes_expected = LEAVE[name]
+    v, surf = make()
+    v, surf = np.ascontiguousarray(v, np.float32), np.ascontiguousarray(surf, np.int32)
+    n = min(200_000, 100_000_000 // len(v))
+    rng = np.random.default_rng(len(v))
+    at = lambda k: np.einsum("ij,ijk->ik", rng.dirichlet((0.6, 0.6, 0.6), n), v[k].astype(float))
+    k = rng.integers(0, len(v), n).astype(np.int32)
+    o = at(k).astype(np.float32)
+    d = rng.standard_normal((n, 3))
+    aimed = rng.random(n) < 0.5
+    d[aimed] = (at(rng.integers(0, len(v), n)) - o)[aimed]
+    d = (d / np.linalg.norm(d, axis=1, keepdims=True)).astype(np.float32)
+    target, t_hit = np.zeros(n, np.int32), np.zeros(n)
+    out, codes, used = np.zeros(n, np.uint8), np.zeros(len(v), np.uint32), C.c_int64()
+    p = {a: x.ctypes.data_as(C.c_void_p) for a, x in
+         dict(v=v, s=surf, o=o, d=d, k=k, target=target, t=t_hit, out=out, codes=codes).items()}
+    lib.nearest_tri(C.c_int64(len(v)), p["v"], p["s"], C.c_int64(n), p["o"], p["d"], p["k"],
+                    p["target"], p["t"])
+    n_proxies = lib.proxy_leave(C.c_int64(len(v)), p["v"], p["s"],
+                                C.c_double(float(np.abs(v).max())), C.c_int64(n), p["o"], p["d"],
+                                p["k"], p["target"], p["t"], p["out"], p["codes"], C.byref(used))
+    assert n_proxies > 0
+    found = set((codes & (SINGLE | APART)).tolist())
+    assert found == codes_expected, found
+    lost = (target != -2) & (out == 0)
+    assert not lost.any(), (int(lost.sum()), n, np.flatnonzero(lost)[:5])
+    assert used.value > n / 20 and (target >= 0).mean() > 0.1 and ((out & 2) == 0).mean() > 0.3
 
 
 def test_meshes_off_any_sphere_or_plane_use_the_bvh(lib):
