@@ -297,9 +297,11 @@ typedef struct rich_trace_opts {
                                (0 or above the occupancy limit -> the limit) */
     int32_t refill_min;     /* refill a warp when at least this many lanes are
                                idle (1..32): the compaction interval (default
-                               32, or 16 in scenes of rectangles alone)      */
+                               32, or 16 in scenes of rectangles alone;
+                               rich_trace_grad 32)                           */
     int32_t chunk;          /* photons a warp takes from the queue at a time
-                               (default 32..128, by what is left)            */
+                               (default 32..128, by what is left;
+                               rich_trace_grad 32)                           */
     int32_t wide_regs;      /* <= 256 threads: 0 caps the trace kernel at 64
                                registers (four blocks per SM), 1 uncapped;
                                257..896 threads: 1 caps it at 72 registers
@@ -312,7 +314,10 @@ typedef struct rich_trace_opts {
     int32_t bvh_smem_nodes; /* top BVH nodes (128 bytes each) staged in shared
                                memory per block by a TMA bulk copy
                                (-1: default, above 256 threads 256, or 16
-                               when the meshes lie on surface proxies)       */
+                               when the meshes lie on surface proxies).
+                               RICH_ERR_ARG for more than fit in shared
+                               memory; with block_threads = 0 blocks of 512
+                               threads hold those that do not fit beside 1024 */
     /* Efficiencies applied before propagation (Sec. 4.3: the quantum
      * efficiency and the mirror reflectivities combined into one
      * accept/reject per photon at its wavelength, and rejected photons not
@@ -418,7 +423,12 @@ RICH_API rich_status rich_set_stream(rich_ctx *ctx, void *stream);
 /* Upload a scene (Sec. 4.1: mirrors and detector as separate surfaces with
  * their own materials; Sec. 4.3: wavelength tables). All pointers in `desc`
  * are HOST memory and are copied. Builds the SAH BVH over the triangles on
- * the host and uploads it. Replaces any previous geometry. Returns
+ * the host and uploads it. When all triangles lie on at most eight spheres or
+ * planes (by surface), grids over those are built and uploaded beside it: about
+ * 550 bytes of device memory per triangle (12 MB for 2.2e4, 82 MB for 1.5e5
+ * triangles), some 100 MB at most, where the BVH and the triangles take 180. The trace
+ * of other scenes walks the BVH and takes about twice as long. Replaces any
+ * previous geometry. Returns
  * RICH_ERR_GEOMETRY for inconsistent descriptions (bad indices, non-finite
  * values, pixel grid not matching a detector rectangle). Synchronous. */
 RICH_API rich_status rich_init_geometry(rich_ctx *ctx, const rich_geometry_desc *desc);
@@ -599,8 +609,8 @@ typedef struct rich_grad_params {
  * sphere tiles moved to theta; every detected photon is then replayed along
  * its recorded reflecting surfaces (fixed topology, the photon's path
  * recomputed per photon, not stored) in forward mode: double-word values
- * (~48 bits), 10 FP32 tangents. The hit (u, v) is smeared by sigma (g1, g2), a Box-Muller pair
- * from the photon's draw block 3; rho = (|(u~, v~) - (cu, cv)| - r) / sigma
+ * (~48 bits), FP32 tangents. The hit (u, v) is smeared by sigma (g1, g2), a
+ * Box-Muller pair from the photon's draw block 3; rho = (|(u~, v~) - (cu, cv)| - r) / sigma
  * and loss = mean rho^2 over the hits whose (track index, plane) target has
  * weight > 0.
  * targets: DEVICE float [n_tracks][n_planes][4] = (cu, cv, r, weight).

@@ -20,8 +20,10 @@
 //                  few spheres or planes are searched through those surfaces
 //                  and a grid of triangle lists, other meshes through a BVH.
 //   k_refine       the detected photons' paths replayed in double-word FP32:
-//                  positions, times, reflection moments and event sums.
-//   k_adjoint      reverse pass of ring moments to the tracks' parameters.
+//                  positions, pixels and event sums.
+//   k_adjoint      gradient of the soft ring chi^2: the detected photons' paths
+//                  replayed with tangents in the tile tilts, the radius of
+//                  curvature and the index.
 #include <climits>
 #include <cstdint>
 #include <cuda_runtime.h>
@@ -921,7 +923,6 @@ __device__ __forceinline__ float disp_tan_f32(const EmitView &em, float omb, flo
 // a dispersive radiator takes tan(theta) of the photon's own wavelength.
 // Isotropic source (the scintillation light named in Sec. 6): the
 // direction is uniform on the sphere, cos(theta) = 1 - 2u from draw block 3.
-template <bool FAR>
 __device__ __forceinline__ void emit_photon(const TrackRec &tr, uint32_t j,
                                             const EmitView &em, const u4 &w0, float lam,
                                             Photon &ph) {
@@ -1009,7 +1010,7 @@ __global__ void __launch_bounds__(256) k_materialize(SceneView sc, EmitView em, 
         Photon ph;
         const uint32_t j = (uint32_t)(g - off);
         const u4 w0 = philox10(0u, j, tr.id, tr.event, em.key0, em.key1);
-        emit_photon<false>(tr, j, em, w0, photon_wavelength<false>(tr, j, em, w0, spec), ph);
+        emit_photon(tr, j, em, w0, photon_wavelength<false>(tr, j, em, w0, spec), ph);
         out.x[g] = ph.o.x;
         out.y[g] = ph.o.y;
         out.z[g] = ph.o.z;
@@ -2214,7 +2215,7 @@ k_trace(TraceArgs A) {
                         if (P.n_prefilter && !(u24f(w0.w) < prefilter_prob(S, P, lam)))
                             rejected = true;
                         else
-                            emit_photon<true>(tr, j, em, w0, lam, ph);
+                            emit_photon(tr, j, em, w0, lam, ph);
                     }
                     if (rejected) {
                         if (ph.g < P.fate_capacity) P.fate[ph.g] = (uint8_t)RICH_FATE_PREFILTERED;

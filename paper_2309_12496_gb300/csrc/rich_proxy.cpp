@@ -23,13 +23,15 @@ using V3 = std::array<double, 3>;
 
 constexpr double kUnit = 1.0 / 16777216.0;   // 2^-24
 constexpr int32_t kNoSurf32 = 0x7FFFFFFF;
-// Cells of 0.12 of the root mean triangle area: most list one triangle. Trace of
-// RICH1, 10^4 tracks, with cells of 0.25, 0.18, 0.12 of it: 458, 442, 428 us; of
-// RICH2, 1.2 x 10^5 tracks: 3.54, 3.42, 3.34 ms (and 835 us, 7.33 ms with cells of
-// the whole of it, before later steps). A cell is at least four margins wide;
-// there are at most kMaxCellsPerTri cells a triangle (meshes whose bounding
-// rectangle is mostly empty get larger cells) and kMaxCells in all (96 MB, which
-// the L2 holds).
+// Cells of kCellScale of the root mean triangle area, at least four margins wide; at
+// most kMaxCellsPerTri cells a triangle and 4096 in a mesh, and kMaxCells in all (96 MB,
+// which the L2 holds). 0.12 of the area is 70 cells a triangle, more where the mesh fills
+// less than its bounding rectangle, so above some 700 triangles the number of cells
+// is what the limit a triangle leaves: 1.43e6 cells on RICH1 (65 a triangle, 11.4 MB),
+// 9.57e6 on RICH2 (64, 76.5 MB); most list one triangle. Trace of RICH1, 10^4 tracks,
+// with 16, 31 and 65 cells a triangle (0.25 and 0.18 of the area, and the limit): 458,
+// 442, 428 us; of RICH2, 1.2 x 10^5 tracks, with 18, 35 and 64: 3.54, 3.42, 3.34 ms (and
+// 835 us, 7.33 ms with one, before later steps). More than 65 were not measured.
 constexpr double kCellScale = 0.12;
 constexpr double kMaxCellsPerTri = 64.0;
 constexpr double kMaxCells = 1.2e7;
